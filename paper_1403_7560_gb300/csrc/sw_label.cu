@@ -11,12 +11,23 @@
 //     bit-planes.
 //   Before it, every site is its own parent in the shared-memory forest; an
 //   x-run is represented by its start, the only site of it ever looked up.
-//   phase 2 (thread per row word): one shared-memory union per pair of runs
-//     joined by +y / +z bonds inside the tile (runs already joined through
+//   phase 2 (thread per row word): the lowest bond of every run to the rows
+//     before it (-y, -z) hooks the run's start there with a plain store: a
+//     start has one parent and every parent a smaller index, so no find and
+//     no atomic is needed.  The other in-tile bonds (a fifth of them at the
+//     critical point) are shared-memory unions (runs already joined through
 //     the previous bit are skipped).
-//   phase 3 (lane per site): find the tile-local root of the site's run
-//     start and write the forest word (root as a global index, local-root
-//     marker, cluster draw).
+//   phase 3 (thread per four sites, or lane per site where L is not a
+//     multiple of 4): find the tile-local root of the site's run start and
+//     write the forest word (root as a global index, local-root marker,
+//     cluster draw).
+//   The kernel is issue-bound (71% of issue slots, 20 of 32 lanes): what
+//   counts is instructions.  A union is two walks and an atomic in a loop the
+//   warp leaves with its slowest thread, so the hooks took the loop from 21 to
+//   8 trips a warp; four sites per thread share the row's loads, address
+//   arithmetic and one 16-byte store.  3D Ising L = 256 at T_c: 85.0 M -> 70.2
+//   M warp instructions, 108.9 -> 87.1 us; from bond planes (XY) 76.2 -> 59.3
+//   us; 2D L = 4096 94.8 -> 76.2 us; 3D L = 100 38.9 -> 29.1 us (ncu, cold L2).
 //   With MEASURE the row threads also measure the incoming spins (the state
 //   after the previous sweep) from the same bytes and equality masks.
 // k_bonds_xy: XY bonds: project on the sweep's mirror axis (once per site,
@@ -136,7 +147,8 @@ struct LabelSmem {
   // Potts, row r's bytes 4j..4j+3 in word j*(ROWS+1)+r (row-thread stores
   // and lane reads both bank-conflict free)
   uint32_t sdraw[kDrawWords];
-  uint32_t sX[ROWS], sS[ROWS];
+  uint32_t sX[ROWS], sY[ROWS];      // bonds along +x inside the word, +y inside the tile
+  uint32_t sZ[S::D == 3 ? ROWS : 1];      // bonds along +z inside the tile
   // Potts histogram: per-warp bins for q <= kSmallQ, shared bins above
   unsigned int s_hist[kHist];
   unsigned int s_whist[kWHist];
@@ -154,7 +166,7 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
   uint32_t* par = sm.par;
   uint32_t* sdraw = sm.sdraw;
   uint32_t* sX = sm.sX;
-  uint32_t* sS = sm.sS;
+  uint32_t* sY = sm.sY;
   unsigned int* s_hist = sm.s_hist;
   unsigned int* s_whist = sm.s_whist;
   long long* s_red = sm.s_red;
@@ -269,29 +281,74 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
     }
   }
   sX[r] = X;
-  sS[r] = S;
+  sY[r] = Y;
+  if (D == 3) sm.sZ[r] = Z;
   __syncthreads();
 
-  // ---- phase 2: unions of runs joined by in-tile +y / +z bonds
+  // ---- phase 2a: the first bond of every x-run to the rows before it hooks
+  // the run's start there (a plain store: each start is written by its own
+  // row's thread only, and its new parent has a smaller index)
   const uint32_t cap = lat.cap;
+  uint32_t Y2 = 0u, Z2 = 0u, Sy = 0u, Sz = 0u;
   if (rowv) {
-    if (Y) {
+    const uint32_t Yp = ry > 0 ? sY[r - 1] : 0u;
+    const uint32_t Zp = (D == 3 && rz > 0) ? sm.sZ[r - TY] : 0u;
+    const uint32_t joined = X << 1;  // bit b: site b is bonded to site b - 1
+    uint32_t both = 0u;
+    if (Yp) {
+      const uint32_t Xn = sX[r - 1];
+      Sy = ~(Xn << 1) & vmask;
+      Y2 = Yp & ~((Yp & X & Xn) << 1);
+    }
+    if (D == 3 && Zp) {
+      const uint32_t Xn = sX[r - TY];
+      Sz = ~(Xn << 1) & vmask;
+      Z2 = Zp & ~((Zp & X & Xn) << 1);
+    }
+    both = Y2 | Z2;
+    // bits above the first one of their run: a carry from each bit runs up
+    // the joined bits and stops at the end of the run
+    const uint32_t seed = (both << 1) & joined;
+    uint32_t F = both & ~((((seed + joined) ^ joined) | seed) & joined);
+    Z2 &= ~(F & ~Y2);
+    const uint32_t FY = F & Y2;
+    Y2 &= ~F;
+    while (F) {
+      const int b = __ffs(F) - 1;
+      F &= F - 1u;
+      const bool y_bond = D == 2 || ((FY >> b) & 1u);
+      par[32 * r + run_start(S, b)] =
+          y_bond ? (uint32_t)(32 * (r - 1)) + run_start(Sy, b) : (uint32_t)(32 * (r - TY)) + run_start(Sz, b);
+    }
+  }
+  __syncthreads();
+
+  // ---- phase 2b: unions for the other in-tile bonds
+  if (rowv) {
+    while (Y2 | Z2) {
+      const bool y_bond = D == 2 || Y2 != 0u;
+      const uint32_t U = y_bond ? Y2 : Z2;
+      const int b = __ffs(U) - 1;
+      if (y_bond) Y2 &= Y2 - 1u;
+      else Z2 &= Z2 - 1u;
+      sunion(par, (uint32_t)(32 * r) + run_start(S, b),
+             y_bond ? (uint32_t)(32 * (r - 1)) + run_start(Sy, b) : (uint32_t)(32 * (r - TY)) + run_start(Sz, b),
+             lat.err, cap);
+    }
+    // bonds around the torus inside the tile (a lattice no longer than it)
+    if (y1 < y && Y) {
       const int rn = r + (y1 - y);
-      const uint32_t Xn = sX[rn], Sn = sS[rn];
-      uint32_t U = Y & ~((Y & X & Xn) << 1);
-      while (U) {
+      const uint32_t Sn = ~(sX[rn] << 1) & vmask;
+      for (uint32_t U = Y; U; U &= U - 1u) {
         const int b = __ffs(U) - 1;
-        U &= U - 1u;
         sunion(par, (uint32_t)(32 * r) + run_start(S, b), (uint32_t)(32 * rn) + run_start(Sn, b), lat.err, cap);
       }
     }
-    if (D == 3 && Z) {
+    if (D == 3 && z1 < z && Z) {
       const int rn = r + TY * (z1 - z);
-      const uint32_t Xn = sX[rn], Sn = sS[rn];
-      uint32_t U = Z & ~((Z & X & Xn) << 1);
-      while (U) {
+      const uint32_t Sn = ~(sX[rn] << 1) & vmask;
+      for (uint32_t U = Z; U; U &= U - 1u) {
         const int b = __ffs(U) - 1;
-        U &= U - 1u;
         sunion(par, (uint32_t)(32 * r) + run_start(S, b), (uint32_t)(32 * rn) + run_start(Sn, b), lat.err, cap);
       }
     }
@@ -302,20 +359,61 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
   // ---- phase 3: forest word of every site
   const uint32_t lr_bit = 1u << lat.sbits;
   const int shift = lat.sbits + 1;
+  const int nrows_y = L - tc.y0, nrows_z = (D == 3) ? L - tc.z0 : 1;  // valid rows (at least)
+  if ((L & 3) == 0) {
+    // a thread per four consecutive sites: their walks advance together, one
+    // 16-byte store
+    const int b0 = 4 * (lane & 7);
+#pragma unroll 1
+    for (int k = 0; k < RPW / 4; ++k) {
+      const int rr = 4 * (warp + NW * k) + (lane >> 3);
+      if (b0 >= nvalid || rr % TY >= nrows_y || rr / TY >= nrows_z) continue;
+      const uint32_t st = ~(sX[rr] << 1);
+      const uint32_t t0 = (uint32_t)(32 * rr + b0);
+      const uint4 own = *reinterpret_cast<const uint4*>(par + t0);
+      uint32_t p[4];
+      p[0] = ((st >> b0) & 1u) ? own.x : par[32 * rr + run_start(st, b0)];
+      p[1] = ((st >> b0) & 2u) ? own.y : p[0];
+      p[2] = ((st >> b0) & 4u) ? own.z : p[1];
+      p[3] = ((st >> b0) & 8u) ? own.w : p[2];
+      uint32_t moved = 1u;  // parents only decrease: at most a walk per site of the tile
+      for (int it = 0; it < ROWS * 32 && moved; ++it) {
+        moved = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t up = par[p[j]];
+          moved |= up ^ p[j];
+          p[j] = up;
+        }
+      }
+      const uint32_t dr = !draws ? 0u
+                          : (two_state || !Smem::kPottsDraws) ? sdraw[rr] >> b0
+                                                              : sdraw[(lane & 7) * (ROWS + 1) + rr];
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t draw = (two_state || !Smem::kPottsDraws) ? (dr >> j) & 1u : (dr >> (8 * j)) & 0xffu;
+        const uint32_t gidx = sm.srow[p[j] >> 5] + (p[j] & 31u);
+        w[j] = (gidx << shift) | (p[j] == t0 + (uint32_t)j ? lr_bit : 0u) | draw;
+      }
+      *reinterpret_cast<uint4*>(lat.forest + sm.srow[rr] + (uint32_t)b0) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  } else {
 #pragma unroll 2
-  for (int k = 0; k < RPW; ++k) {
-    const int rr = warp + NW * k;
-    const uint32_t st = sS[rr];
-    if (st == 0u || lane >= nvalid) continue;
-    const uint32_t t = (uint32_t)(32 * rr + lane);
-    const uint32_t lr = sfind(par, (uint32_t)(32 * rr) + run_start(st, lane));
-    const uint32_t gidx = sm.srow[lr >> 5] + (lr & 31u);
-    const uint32_t i = sm.srow[rr] + (uint32_t)lane;
-    const uint32_t draw = !draws ? 0u
-                          : (two_state || !Smem::kPottsDraws)
-                              ? (sdraw[rr] >> lane) & 1u
-                              : (sdraw[(lane >> 2) * (ROWS + 1) + rr] >> (8 * (lane & 3))) & 0xffu;
-    lat.forest[i] = (gidx << shift) | (lr == t ? lr_bit : 0u) | draw;
+    for (int k = 0; k < RPW; ++k) {
+      const int rr = warp + NW * k;
+      if (lane >= nvalid || rr % TY >= nrows_y || rr / TY >= nrows_z) continue;
+      const uint32_t st = ~(sX[rr] << 1);
+      const uint32_t t = (uint32_t)(32 * rr + lane);
+      const uint32_t lr = sfind(par, (uint32_t)(32 * rr) + run_start(st, lane));
+      const uint32_t gidx = sm.srow[lr >> 5] + (lr & 31u);
+      const uint32_t i = sm.srow[rr] + (uint32_t)lane;
+      const uint32_t draw = !draws ? 0u
+                            : (two_state || !Smem::kPottsDraws)
+                                ? (sdraw[rr] >> lane) & 1u
+                                : (sdraw[(lane >> 2) * (ROWS + 1) + rr] >> (8 * (lane & 3))) & 0xffu;
+      lat.forest[i] = (gidx << shift) | (lr == t ? lr_bit : 0u) | draw;
+    }
   }
   if (MEASURE) {
     if (MM == 2) {
