@@ -40,10 +40,11 @@ struct sw_batch {
   int shape = 0;                      // tile shape (index into the shape table)
   int schedule = 0;                   // label layout (bit 0) and grid form (bit 1)
   // small members (whole sweeps in one CTA's shared memory): member indices,
-  // the Ising ones then the Potts ones, run on a forked branch of the graph
+  // run beside the graph's replays on a stream of their own
   uint32_t* d_small = nullptr;
   size_t cap_small = 0;
-  uint32_t n_small_ising = 0, n_small_potts = 0;
+  uint32_t n_small = 0;
+  size_t small_smem = 0;              // the largest small member's shared memory
   std::vector<bool> is_small;         // per member
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -52,6 +53,8 @@ struct sw_batch {
 };
 
 namespace {
+
+constexpr uint32_t kSmallChunk = 256;  // sweeps of the small members per launch
 
 int bfail(int code, const std::string& msg) {
   swgb::set_last_error(msg);
@@ -94,13 +97,15 @@ size_t member_tiles(const sw_batch* b, const sw_handle* h) {
 // or configuration.
 int rebuild(sw_batch* b) {
   size_t ntiles = 0;
-  std::vector<uint32_t> small_ising, small_potts;
+  std::vector<uint32_t> small;
+  size_t small_smem = 0;
   b->is_small.assign(b->members.size(), false);
   for (size_t m = 0; m < b->members.size(); ++m) {
     sw_handle* h = b->members[m];
     if (swgb::small_lattice(h->lat)) {
       b->is_small[m] = true;
-      (h->model == SW_POTTS ? small_potts : small_ising).push_back((uint32_t)m);
+      small.push_back((uint32_t)m);
+      small_smem = std::max(small_smem, swgb::small_layout_bytes(h->lat));
     } else {
       ntiles += member_tiles(b, h);
     }
@@ -127,7 +132,7 @@ int rebuild(sw_batch* b) {
       return bfail(SW_ERR_OOM, std::string("batch tile map: ") + cudaGetErrorString(e));
     b->cap_tiles = cap;
   }
-  const size_t nsmall = small_ising.size() + small_potts.size();
+  const size_t nsmall = small.size();
   if (nsmall > b->cap_small) {
     swgb::dev_free(b->d_small, b->stream);
     b->d_small = nullptr;
@@ -136,13 +141,11 @@ int rebuild(sw_batch* b) {
       return bfail(SW_ERR_OOM, std::string("batch small-member list: ") + cudaGetErrorString(e));
     b->cap_small = cap;
   }
-  // the (re)allocations above are ordered on the batch stream; the copies
-  // below run on the legacy stream
-  if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return bcuda(e, "batch sync");
+  // the copies below run on the batch stream, whose kernels (and the side
+  // stream's, after ev_fork) read them: a copy from pageable memory on
+  // another stream may still be in flight when the call returns
   if (nsmall) {
-    std::vector<uint32_t> all(small_ising);
-    all.insert(all.end(), small_potts.begin(), small_potts.end());
-    if ((e = cudaMemcpy(b->d_small, all.data(), nsmall * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(b->d_small, small.data(), nsmall * 4, cudaMemcpyHostToDevice, b->stream)) != cudaSuccess)
       return bcuda(e, "batch small-member list");
     if (!b->side) {
       if ((e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking)) != cudaSuccess ||
@@ -150,10 +153,9 @@ int rebuild(sw_batch* b) {
           (e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming)) != cudaSuccess)
         return bcuda(e, "batch side stream");
     }
-    if ((e = swgb::prepare_small_batch()) != cudaSuccess) return bcuda(e, "small-lattice kernels");
   }
-  b->n_small_ising = (uint32_t)small_ising.size();
-  b->n_small_potts = (uint32_t)small_potts.size();
+  b->n_small = (uint32_t)nsmall;
+  b->small_smem = small_smem;
   std::vector<uint32_t> lat(ntiles), idx(ntiles);
   size_t t = 0;
   for (int pass = 0; pass < 2; ++pass) {  // Ising members' tiles, then Potts
@@ -169,37 +171,26 @@ int rebuild(sw_batch* b) {
     if (pass == 0) b->ising_tiles = (uint32_t)t;
   }
   if (ntiles) {
-    if ((e = cudaMemcpy(b->d_tiles, lat.data(), ntiles * 4, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(b->d_tiles + b->cap_tiles, idx.data(), ntiles * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(b->d_tiles, lat.data(), ntiles * 4, cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(b->d_tiles + b->cap_tiles, idx.data(), ntiles * 4, cudaMemcpyHostToDevice, b->stream)) !=
+            cudaSuccess)
       return bcuda(e, "batch tile map");
   }
+  // the lists on the host go out of scope with this call
+  if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return bcuda(e, "batch sync");
   b->ntiles = (uint32_t)ntiles;
   drop_graph(b);
-  if (ntiles || nsmall) {
-    // capture one sweep: the small members on a forked branch; labels (+
-    // measurement), merge, compression, apply of the tiled ones; the step
+  if (ntiles) {
+    // capture one sweep of the tiled members: labels (+ measurement), merge,
+    // compression, apply; the step
     cudaGraph_t g = nullptr;
     const BatchView v = view(b);
     e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaError_t le = cudaSuccess;
-      if (nsmall) {
-        le = cudaEventRecord(b->ev_fork, b->stream);
-        if (le == cudaSuccess) le = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
-        if (le == cudaSuccess)
-          le = swgb::launch_small_batch(v, b->dim, b->d_small, b->n_small_ising, b->d_small + b->n_small_ising,
-                                        b->n_small_potts, b->side);
-        if (le == cudaSuccess) le = cudaEventRecord(b->ev_join, b->side);
-      }
-      if (le == cudaSuccess && ntiles) {
-        le = swgb::launch_label_batch(v, b->dim, b->shape, b->schedule, b->ising_tiles, b->ntiles - b->ising_tiles,
-                                      b->stream);
-        if (le == cudaSuccess)
-          le = swgb::launch_merge_batch(v, b->dim, b->shape, b->schedule, b->ntiles, b->stream);
-        if (le == cudaSuccess)
-          le = swgb::launch_flip_batch(v, b->dim, b->shape, b->schedule, b->ntiles, b->stream);
-      }
-      if (le == cudaSuccess && nsmall) le = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+      cudaError_t le = swgb::launch_label_batch(v, b->dim, b->shape, b->schedule, b->ising_tiles,
+                                                b->ntiles - b->ising_tiles, b->stream);
+      if (le == cudaSuccess) le = swgb::launch_merge_batch(v, b->dim, b->shape, b->schedule, b->ntiles, b->stream);
+      if (le == cudaSuccess) le = swgb::launch_flip_batch(v, b->dim, b->shape, b->schedule, b->ntiles, b->stream);
       if (le == cudaSuccess) le = swgb::launch_advance(v, b->stream);
       e = cudaStreamEndCapture(b->stream, &g);
       if (e == cudaSuccess) e = le;
@@ -368,7 +359,17 @@ int batch_sweep(sw_batch* b, int n, float* ms) {
       return bcuda(e, "batch timing");
     }
   }
-  for (uint32_t s = 0; s < replays && e == cudaSuccess; ++s) e = cudaGraphLaunch(b->graph, b->stream);
+  // the small members' sweeps, many per launch, beside the replays
+  if (b->n_small) {
+    e = cudaEventRecord(b->ev_fork, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
+    for (uint32_t s = 0; s < replays && e == cudaSuccess; s += kSmallChunk)
+      e = swgb::launch_small_batch(b->d_members, b->dim, b->d_small, b->n_small, b->small_smem, s, kSmallChunk,
+                                   b->side);
+    if (e == cudaSuccess) e = cudaEventRecord(b->ev_join, b->side);
+  }
+  for (uint32_t s = 0; b->ntiles && s < replays && e == cudaSuccess; ++s) e = cudaGraphLaunch(b->graph, b->stream);
+  if (e == cudaSuccess && b->n_small) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
   if (e == cudaSuccess && ms) e = cudaEventRecord(t1, b->stream);
   // later work on each member waits for the batch
   if (e == cudaSuccess) e = cudaEventRecord(b->ev, b->stream);

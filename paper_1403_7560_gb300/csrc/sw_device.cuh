@@ -95,6 +95,30 @@ __device__ __forceinline__ uint32_t bernoulli_word(uint32_t g, uint32_t sweep, i
   return lt;
 }
 
+// cmp_step with the threshold bit as a lane's mask (0 or all ones).
+__device__ __forceinline__ void cmp_step_lane(uint32_t& lt, uint32_t& eq, uint32_t r, int tmask) {
+  const uint32_t tm = (uint32_t)tmask;
+  lt |= eq & ~r & tm;
+  eq &= ~(r ^ tm);
+}
+
+// The rest of a Bernoulli word from call c0 on, for the lanes in `live`.
+__device__ __forceinline__ uint32_t bernoulli_tail(uint32_t g, uint32_t sweep, int d, uint32_t t, uint32_t live,
+                                                   const uint32_t* rk, int c0) {
+  uint32_t lt = 0u, eq = live;
+#pragma unroll 1
+  for (int c = c0; c < 8; ++c) {
+    const uint4 w = philox(g, sweep, kBond, (uint32_t)(8 * d + c), rk);
+    const uint32_t tb = t << (4 * c);
+    cmp_step_lane(lt, eq, w.x, (int)tb >> 31);
+    cmp_step_lane(lt, eq, w.y, (int)(tb << 1) >> 31);
+    cmp_step_lane(lt, eq, w.z, (int)(tb << 2) >> 31);
+    cmp_step_lane(lt, eq, w.w, (int)(tb << 3) >> 31);
+    if (eq == 0u) break;
+  }
+  return lt;
+}
+
 // Cluster draw value of a site from its 32-bit draw word w: floor(w q / 2^32)
 // (Ising and XY use q = 2: 1 = flip to -1 / reflect).
 __device__ __forceinline__ uint32_t draw_value(uint32_t w, uint32_t q) {
@@ -414,13 +438,11 @@ __device__ __forceinline__ void finalize_record(const Lattice& lat, const Measur
   commit_record<NW>(lat, mb, sweep, M, E, S2, mx, my, exy, s_ri);
 }
 
-// The record of `sweep` from its sums and cluster count, and the update of
-// the FP64 accumulators acc[6] (global, or a shared copy).  Called by one
-// thread.
-__device__ __forceinline__ void write_record(const Lattice& lat, const Measure& mb, uint32_t sweep,
+// The record of `sweep` from its sums and cluster count; its M2 and E go to
+// M2 and Ed.  Called by one thread.
+__device__ __forceinline__ void store_record(const Lattice& lat, const Measure& mb, uint32_t sweep,
                                              long long M, long long E, long long S2, double mx, double my,
-                                             double exy, long long ncl, double* acc) {
-  double M2, Ed;
+                                             double exy, long long ncl, double& M2, double& Ed) {
   if (lat.model == kIsing) {
     M2 = __dmul_rn((double)M, (double)M);
     Ed = (double)E;
@@ -443,6 +465,15 @@ __device__ __forceinline__ void write_record(const Lattice& lat, const Measure& 
   rec->e_xy = exy;
   rec->M2 = M2;
   rec->Ed = Ed;
+}
+
+// The record of `sweep` and the update of the FP64 accumulators acc[6].
+// Called by one thread.
+__device__ __forceinline__ void write_record(const Lattice& lat, const Measure& mb, uint32_t sweep,
+                                             long long M, long long E, long long S2, double mx, double my,
+                                             double exy, long long ncl, double* acc) {
+  double M2, Ed;
+  store_record(lat, mb, sweep, M, E, S2, mx, my, exy, ncl, M2, Ed);
   acc[0] = __dadd_rn(acc[0], 1.0);
   acc[1] = __dadd_rn(acc[1], M2);
   acc[2] = __dadd_rn(acc[2], __dmul_rn(M2, M2));

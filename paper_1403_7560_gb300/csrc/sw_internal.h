@@ -231,13 +231,12 @@ unsigned batch_grid(K* k, int threads, uint32_t n) {
 }
 // Advances the batch step counter (after every member's sweep).
 cudaError_t launch_advance(const BatchView& bv, cudaStream_t st);
-// Small members of a batch (sw_small.cu): one CTA per member, whole sweeps
-// in shared memory; lists of member indices, Ising and Potts.
-// prepare_small_batch sets the kernels' shared-memory limit (once, before
-// capture).
-cudaError_t prepare_small_batch();
-cudaError_t launch_small_batch(const BatchView& bv, int dim, const uint32_t* ising_list, uint32_t n_ising,
-                               const uint32_t* potts_list, uint32_t n_potts, cudaStream_t st);
+// Small members of a batch (sw_small.cu): one CTA per member of the list (of
+// member indices), whole sweeps in `smem` bytes of shared memory (the largest
+// member's small_layout_bytes): up to n sweeps each from sweep `first` of the
+// current batch call.
+cudaError_t launch_small_batch(const BatchMember* members, int dim, const uint32_t* list, uint32_t count,
+                               size_t smem, uint32_t first, uint32_t n, cudaStream_t st);
 
 // Write the record of a pending measured sweep of h (stand-alone kernel).
 cudaError_t flush_pending(struct ::sw_handle* h);
@@ -246,11 +245,12 @@ size_t handle_block_bytes();
 // Small Ising/Potts lattices (sw_small.cu): whole sweeps by one CTA with
 // the lattice in shared memory, n sweeps per launch, records written as
 // the tiled path writes them.
-constexpr int kSmallSites = 8192;  // the shared-memory layout's capacity
+constexpr uint32_t kSmallSites2D = 8192, kSmallSites3D = 4096;
+// Dynamic shared memory a small lattice may take (227 KB a CTA less the
+// static part).
+constexpr size_t kSmallSharedBytes = 192 * 1024;
 size_t small_layout_bytes_max();
-// Largest lattice (sites) that takes the one-CTA path: 2D Ising 4096, 2D
-// Potts 8192, 3D 1024 (where it beats the tiled path).
-uint32_t small_sites_limit(int model, int dim);
+size_t small_layout_bytes(const Lattice& lat);
 bool small_lattice(const Lattice& lat);
 cudaError_t launch_sweeps_small(const Lattice& lat, const Measure& m, uint32_t sweep0, int n, bool measure,
                                 cudaStream_t st);

@@ -34,3 +34,63 @@ def test_tile_labels_at_tile_edges(sw, dim, L):
             assert np.array_equal(sw.sw_label_from_bonds(h, m), oracle.labels(dim, L, m)), density
     finally:
         sw.sw_destroy(h)
+
+
+@pytest.mark.parametrize("model,dim,L,q", [
+    (ISING, 2, 4, 2), (ISING, 2, 5, 2), (ISING, 2, 31, 2), (ISING, 2, 32, 2), (ISING, 2, 33, 2), (ISING, 2, 65, 2),
+    (ISING, 2, 90, 2), (ISING, 3, 4, 2), (ISING, 3, 7, 2), (ISING, 3, 16, 2),
+    (POTTS, 2, 6, 2), (POTTS, 2, 33, 3), (POTTS, 2, 90, 5), (POTTS, 2, 64, 16), (POTTS, 2, 37, 17),
+    (POTTS, 2, 90, 256), (POTTS, 3, 5, 4), (POTTS, 3, 16, 3)])
+def test_one_cta_sweeps(sw, model, dim, L, q):
+    """Whole sweeps in shared memory: calls longer than the record ring (64
+    sweeps), bonds, labels, states, records and accumulators."""
+    T = 2.3 if model == ISING and dim == 2 else 4.5 if model == ISING else 0.9
+    h = sw.sw_create(model, dim, L, q, T, 77 + L)
+    o = oracle.Oracle(model, dim, L, q, T, 77 + L)
+    try:
+        sw.sw_sweep(h, 130)
+        sw.sw_discard(h, 3)
+        sw.sw_sweep(h, 64)
+        recs = []
+        for k in range(197):
+            o.sweep(1, measure=not 130 <= k < 133)
+            recs.append(o.last_record())
+        assert np.array_equal(sw.sw_get_spins(h), o.spins)
+        assert np.array_equal(sw.sw_get_bonds(h), o.planes)
+        assert np.array_equal(sw.sw_get_labels(h), o.labels)
+        for first, n in ((1, 130), (134, 64)):
+            for r, ref in zip(sw.sw_get_series(h, first, n), recs[first - 1:]):
+                assert all(r[f] == ref[f] for f in ref if f in r), (r, ref)
+        got, ref = sw.sw_measure(h), o.take_acc()
+        assert all(got[f] == ref[f] for f in ref)
+    finally:
+        sw.sw_destroy(h)
+        o.close()
+
+
+def test_small_members_over_several_launches(sw):
+    """More sweeps in a batch call than one launch of the small members takes,
+    with members that stop early, beside a tiled member."""
+    spec = [(ISING, 2, 8, 2, 2.3, 1, 0), (POTTS, 2, 13, 3, 1.0, 2, 300), (ISING, 2, 33, 2, 2.2, 3, 10),
+            (ISING, 2, 100, 2, 2.27, 4, 5)]
+    b = sw.sw_batch_create(2)
+    hs = [sw.sw_create(*s[:6]) for s in spec]
+    try:
+        for h, s in zip(hs, spec):
+            sw.sw_batch_add(b, h)
+            if s[6]:
+                sw.sw_set_sweep_target(h, s[6])
+        sw.sw_batch_sweep(b, 600)
+        for h, s in zip(hs, spec):
+            n = s[6] or 600
+            o = oracle.Oracle(*s[:6])
+            o.sweep(n)
+            assert sw.sw_sweep_counter(h) == n
+            assert np.array_equal(sw.sw_get_spins(h), o.spins)
+            got, ref = sw.sw_measure(h), o.take_acc()
+            assert all(got[f] == ref[f] for f in ref), s
+            o.close()
+    finally:
+        sw.sw_batch_destroy(b)
+        for h in hs:
+            sw.sw_destroy(h)
