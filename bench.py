@@ -571,7 +571,7 @@ def _job_list(specs):
 
 
 def batch_launches(specs, schedule):
-    """Kernels one batch sweep launches: the tiled members' labels (one
+    """Kernels of one batch sweep, a launch per phase: the tiled members' labels (one
     launch per model under label layout 0, one in all under layout 1 -- bit 0
     of the schedule), merge (one launch, or one per axis under bit 2),
     compression and apply; one launch per model of the small members (2D up
@@ -584,6 +584,16 @@ def batch_launches(specs, schedule):
     dim = specs[0][1] if specs else 2
     merges = (dim if schedule & 4 else 1) if tiled else 0
     return labels + (merges + 2 if tiled else 0) + len(small) + 1
+
+
+def batch_call_launches(specs, schedule, sweeps):
+    """Kernels one sw_batch_sweep(b, sweeps) launches: per sweep the tiled
+    members' labels, merge, compression, apply and the step counter
+    (batch_launches without small members); for the small members (2D up to
+    12544 sites, 3D up to 10648) one launch per 256 sweeps."""
+    tiled = [x for x in specs if x[2] ** x[1] > (12544 if x[1] == 2 else 10648)]
+    n = batch_launches(tiled, schedule) * sweeps if tiled else 0
+    return n + (-(-sweeps // 256) if len(tiled) < len(specs) else 0)
 
 
 def small_batch(sw, inputs, st, sweeps=50):
@@ -622,7 +632,7 @@ def small_batch(sw, inputs, st, sweeps=50):
             "ms_per_step": 1e3 * t_batch / sweeps,
             "serial": {"value": sites * sweeps / (t_serial * 1e9), "unit": UNIT},
             "speedup_vs_serial": t_serial / t_batch,
-            "gpu_launches": batch_launches(specs, 0) * sweeps}
+            "gpu_launches": batch_call_launches(specs, 0, sweeps)}
 
 
 def batch_leg(args, st):
@@ -690,7 +700,7 @@ def batch_leg(args, st):
                                                          for sc in range(tune_ms.shape[1]) if tune_ms[sh, sc] > 0},
                          "note": "5 timed sweeps per configuration, before the timed region"},
             "small_lattices": small,
-            "gpu_launches": batch_launches(specs, cfg["schedule"]) * args.batch_sweeps, "clocks": clk}
+            "gpu_launches": batch_call_launches(specs, cfg["schedule"], args.batch_sweeps), "clocks": clk}
 
 
 def run_batch(args):

@@ -360,7 +360,7 @@ sw_handle* sw_create(int model, int dim, int L, int q, double T, uint64_t seed) 
   const size_t block_bytes = bl.total;
 
   cudaStream_t st = h->stream;
-  if ((e = swgb::dev_alloc(&lat.spins, h->spin_bytes, st)) != cudaSuccess ||
+  if ((e = swgb::dev_alloc(&lat.spins, h->spin_bytes + swgb::kSpinPad, st)) != cudaSuccess ||
       (e = swgb::dev_alloc((void**)&lat.planes, h->bond_words * 4, st)) != cudaSuccess ||
       (e = swgb::dev_alloc((void**)&lat.forest, (size_t)N * 4, st)) != cudaSuccess ||
       (e = swgb::dev_alloc((void**)&lat.hooked, hook_words * 4, st)) != cudaSuccess ||

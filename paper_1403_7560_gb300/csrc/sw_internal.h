@@ -97,6 +97,10 @@ struct BatchView {
   uint32_t* step;
 };
 
+// Bytes behind the states of every spin buffer: the row loads read whole
+// words past the last row's end.
+constexpr size_t kSpinPad = 64;
+
 // Record layout written by the measurement kernel (mirrors sw_record).
 struct Record {
   unsigned long long sweep;
@@ -245,7 +249,12 @@ size_t handle_block_bytes();
 // Small Ising/Potts lattices (sw_small.cu): whole sweeps by one CTA with
 // the lattice in shared memory, n sweeps per launch, records written as
 // the tiled path writes them.
-constexpr uint32_t kSmallSites2D = 8192, kSmallSites3D = 4096;
+// the limits are where the one-CTA path stops beating the tiled one with its
+// split labeling (us per sweep at T_c, one CTA / tiled): 2D Ising L = 96 13.8 /
+// 18.8, 112 17.9 / 18.6, 128 19.5 / 20.4, 2D Potts q = 3 L = 128 23.4 / 22.7;
+// 3D Ising L = 18 14.4 / 23.8, 20 17.7 / 24.9 (beyond 22 the shared memory
+// does not hold it).
+constexpr uint32_t kSmallSites2D = 12544, kSmallSites3D = 10648;
 // Dynamic shared memory a small lattice may take (227 KB a CTA less the
 // static part).
 constexpr size_t kSmallSharedBytes = 192 * 1024;

@@ -43,7 +43,7 @@ cudaError_t ensure_io(sw_handle* h) {
   if (h->io_in) return cudaSuccess;
   cudaError_t e = cudaStreamCreateWithFlags(&h->io_in, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->io_out, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = swgb::dev_alloc(&h->stage_in, h->spin_bytes, h->stream);
+  if (e == cudaSuccess) e = swgb::dev_alloc(&h->stage_in, h->spin_bytes + swgb::kSpinPad, h->stream);
   // the copy streams use the buffers: order them after the allocations
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   cudaEvent_t* evs[6] = {&h->ev_in_done, &h->ev_in_free, &h->ev_state, &h->ev_rec, &h->ev_down[0], &h->ev_down[1]};

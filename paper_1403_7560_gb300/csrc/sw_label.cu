@@ -45,52 +45,66 @@ constexpr int kSmallQ = 16;  // Potts histograms up to this q are counted per th
 
 // The 32 spin bytes of a row word and of its +x, +y, +z neighbour words.
 struct RowBytes {
-  uint32_t a[8], ax[8], ay[8], az[8];
+  uint32_t a[9], ax[8], ay[8], az[8];
 };
 
-template <int D>
-__device__ __forceinline__ void load_rows(const uint8_t* s, int L, int x0, uint32_t row,
-                                          uint32_t row_y, uint32_t row_z, RowBytes& rb) {
-  const uint32_t base = row * (uint32_t)L + (uint32_t)x0;
-  if ((L & 31) == 0) {
-    // 32-byte aligned rows: two 16-byte loads per row word
+// The 32 bytes from s[base] on as 8 words (and w[8], whose low byte is byte
+// 32), whatever the alignment: two 16-byte loads where every row is 16-byte
+// aligned (L a multiple of 16), else aligned words shifted into place (against
+// a byte load per site: 2D L = 515 sweeps 39.7 -> 32.2 us, 3D L = 100 46.3 ->
+// 41.5, the labeling unsplit).  Up to 36 bytes from s[base] are read: past the row's end they belong to the next row, past
+// the lattice's to the buffer's padding (kSpinPad), and the caller masks them.
+template <bool NEXT>
+__device__ __forceinline__ void load32(const uint8_t* s, uint32_t base, bool vec16, uint32_t* w) {
+  if (vec16) {
     const uint4* p = reinterpret_cast<const uint4*>(s + base);
-    const uint4* py = reinterpret_cast<const uint4*>(s + row_y * (uint32_t)L + (uint32_t)x0);
-    uint4 v0 = __ldg(p), v1 = __ldg(p + 1);
-    rb.a[0] = v0.x; rb.a[1] = v0.y; rb.a[2] = v0.z; rb.a[3] = v0.w;
-    rb.a[4] = v1.x; rb.a[5] = v1.y; rb.a[6] = v1.z; rb.a[7] = v1.w;
-    v0 = __ldg(py); v1 = __ldg(py + 1);
-    rb.ay[0] = v0.x; rb.ay[1] = v0.y; rb.ay[2] = v0.z; rb.ay[3] = v0.w;
-    rb.ay[4] = v1.x; rb.ay[5] = v1.y; rb.ay[6] = v1.z; rb.ay[7] = v1.w;
-    if (D == 3) {
-      const uint4* pz = reinterpret_cast<const uint4*>(s + row_z * (uint32_t)L + (uint32_t)x0);
-      v0 = __ldg(pz); v1 = __ldg(pz + 1);
-      rb.az[0] = v0.x; rb.az[1] = v0.y; rb.az[2] = v0.z; rb.az[3] = v0.w;
-      rb.az[4] = v1.x; rb.az[5] = v1.y; rb.az[6] = v1.z; rb.az[7] = v1.w;
-    }
-    // +x neighbours: the row shifted by one byte; the last one wraps to x = 0
-    const uint32_t nx = (x0 + 32 < L) ? s[base + 32] : s[row * (uint32_t)L];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) rb.ax[k] = __byte_perm(rb.a[k], rb.a[k + 1], 0x4321);
-    rb.ax[7] = __byte_perm(rb.a[7], nx, 0x4321);
+    const uint4 v0 = __ldg(p), v1 = __ldg(p + 1);
+    w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w;
+    w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w;
+    if (NEXT) w[8] = __ldg(s + base + 32);
   } else {
-    // general L: byte loads of the valid sites, zero elsewhere
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(s + (base & ~3u));
+    const uint32_t sh = 8u * (base & 3u);
+    uint32_t v = __ldg(p);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) rb.a[k] = rb.ax[k] = rb.ay[k] = rb.az[k] = 0u;
-    const uint32_t rowL = row * (uint32_t)L, rowyL = row_y * (uint32_t)L, rowzL = row_z * (uint32_t)L;
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t v1 = __ldg(p + k + 1);
+      w[k] = __funnelshift_r(v, v1, sh);
+      v = v1;
+    }
+    if (NEXT) w[8] = v >> sh;
+  }
+}
+
+// A row word's bytes moved by one site along +x; w[8] holds byte 32.  The last
+// site of the row has the row's first one as its neighbour.
+__device__ __forceinline__ void shift_row(const uint8_t* s, uint32_t* w, uint32_t row_start, int L, int x0,
+                                          int nvalid, uint32_t* ax) {
+  const bool row_end = x0 + 32 >= L;
+  const uint32_t first = row_end ? (uint32_t)__ldg(s + row_start) : 0u;
+  if (row_end && nvalid == 32) w[8] = first;
 #pragma unroll
-    for (int b = 0; b < 32; ++b) {
-      const int x = x0 + b;
-      if (x < L) {
-        const int x1 = (x + 1 == L) ? 0 : x + 1;
-        const int sh = 8 * (b & 3);
-        rb.a[b >> 2] |= (uint32_t)s[rowL + x] << sh;
-        rb.ax[b >> 2] |= (uint32_t)s[rowL + x1] << sh;
-        rb.ay[b >> 2] |= (uint32_t)s[rowyL + x] << sh;
-        if (D == 3) rb.az[b >> 2] |= (uint32_t)s[rowzL + x] << sh;
-      }
+  for (int k = 0; k < 8; ++k) ax[k] = __byte_perm(w[k], w[k + 1], 0x4321);
+  if (row_end && nvalid < 32) {
+    const int at = nvalid - 1;
+    const uint32_t byte = 0xffu << (8 * (at & 3)), rep = first * 0x01010101u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t m = (at >> 2) == k ? byte : 0u;
+      ax[k] = (ax[k] & ~m) | (rep & m);
     }
   }
+}
+
+template <int D>
+__device__ __forceinline__ void load_rows(const uint8_t* s, int L, int x0, int nvalid, uint32_t row,
+                                          uint32_t row_y, uint32_t row_z, RowBytes& rb) {
+  const bool vec16 = (L & 15) == 0;
+  const uint32_t rowL = row * (uint32_t)L;
+  load32<true>(s, rowL + (uint32_t)x0, vec16, rb.a);
+  load32<false>(s, row_y * (uint32_t)L + (uint32_t)x0, vec16, rb.ay);
+  if (D == 3) load32<false>(s, row_z * (uint32_t)L + (uint32_t)x0, vec16, rb.az);
+  shift_row(s, rb.a, rowL, L, x0, nvalid, rb.ax);
 }
 
 // Measurement of one 32-site row word from its bytes and the equality masks
@@ -98,33 +112,38 @@ __device__ __forceinline__ void load_rows(const uint8_t* s, int L, int x0, uint3
 // E = -(#parallel - #antiparallel) over the +d bonds.  MM 2 (Potts): E = the
 // number of unequal +d bonds, and the histogram n[k] of the states (per-warp
 // bins for q <= kSmallQ, shared bins above).
-template <int D, int MM>
-__device__ __forceinline__ void measure_row(const RowBytes& rb, uint32_t e0, uint32_t e1, uint32_t e2,
-                                            uint32_t vmask, int nvalid, int q, int& m_acc, int& e_acc,
-                                            unsigned int* warp_hist, unsigned int* s_hist) {
-  const int par_bonds = __popc(e0) + __popc(e1) + (D == 3 ? __popc(e2) : 0);
+template <int MM>
+__device__ __forceinline__ void measure_state(const uint32_t* a, uint32_t vmask, int nvalid, int q, int& m_acc,
+                                              unsigned int* warp_hist, unsigned int* s_hist) {
   if (MM == 1) {
     uint32_t ones[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) ones[k] = 0x01010101u;
-    m_acc += 2 * __popc(eq_bits(rb.a, ones) & vmask) - nvalid;
-    e_acc -= 2 * par_bonds - D * nvalid;
+    m_acc += 2 * __popc(eq_bits(a, ones) & vmask) - nvalid;
   } else if (MM == 2) {
-    e_acc += D * nvalid - par_bonds;
     if (q <= kSmallQ) {
       for (int k = 0; k < q; ++k) {
         uint32_t kk[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) kk[j] = 0x01010101u * (uint32_t)k;
-        const unsigned c = (unsigned)__popc(eq_bits(rb.a, kk) & vmask);
+        const unsigned c = (unsigned)__popc(eq_bits(a, kk) & vmask);
         if (c) atomicAdd(&warp_hist[k], c);
       }
     } else {
 #pragma unroll
       for (int b = 0; b < 32; ++b)
-        if (b < nvalid) atomicAdd(&s_hist[(rb.a[b >> 2] >> (8 * (b & 3))) & 0xffu], 1u);
+        if (b < nvalid) atomicAdd(&s_hist[(a[b >> 2] >> (8 * (b & 3))) & 0xffu], 1u);
     }
   }
+}
+
+template <int D, int MM>
+__device__ __forceinline__ void measure_row(const RowBytes& rb, uint32_t e0, uint32_t e1, uint32_t e2,
+                                            uint32_t vmask, int nvalid, int q, int& m_acc, int& e_acc,
+                                            unsigned int* warp_hist, unsigned int* s_hist) {
+  const int par_bonds = __popc(e0) + __popc(e1) + (D == 3 ? __popc(e2) : 0);
+  e_acc += D * nvalid - (MM == 1 ? 2 : 1) * par_bonds;
+  measure_state<MM>(rb.a, vmask, nvalid, q, m_acc, warp_hist, s_hist);
 }
 
 // MM (measurement mode) 1 = Ising, 2 = Potts: also measure the incoming
@@ -135,9 +154,9 @@ __device__ __forceinline__ void measure_row(const RowBytes& rb, uint32_t e0, uin
 // or Potts (3) cluster draws.
 // Shared memory of one tile's labeling in measurement mode MM (the Potts
 // draw words and histograms only where Potts lattices can run).
-template <class S, int MM>
+template <class S, int MM, int K = 1>
 struct LabelSmem {
-  static constexpr int ROWS = S::ROWS, NW = S::THREADS / 32;
+  static constexpr int ROWS = S::ROWS, NW = K * S::THREADS / 32;
   static constexpr bool kPottsDraws = MM >= 2;  // MM 0 and 1: two-state draws only
   static constexpr int kDrawWords = (kPottsDraws ? 8 : 1) * (ROWS + 1);
   static constexpr int kHist = MM == 2 ? 256 : 1, kWHist = MM == 2 ? NW * kSmallQ : 1;
@@ -155,13 +174,13 @@ struct LabelSmem {
   long long s_red[NW];
 };
 
-template <class Sh, bool FROM_MASK, int MM, class Smem>
+template <class Sh, int K, bool FROM_MASK, int MM, class Smem>
 __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, uint32_t sweep,
                                            const Measure& mb, Smem& sm) {
   constexpr bool MEASURE = MM == 1 || MM == 2;
-  constexpr int D = Sh::D, TY = Sh::TY, TZ = Sh::TZ, ROWS = Sh::ROWS, NT = Sh::THREADS;
+  constexpr int D = Sh::D, TY = Sh::TY, TZ = Sh::TZ, ROWS = Sh::ROWS, NT = K * Sh::THREADS;
   constexpr int NW = NT / 32, RPW = ROWS / NW;
-  static_assert(ROWS == NT && NT % 32 == 0, "one thread per row word, whole warps");
+  static_assert(ROWS == Sh::THREADS && ROWS % 32 == 0, "K threads per row word, whole warps");
   static_assert(!(MEASURE && FROM_MASK), "measurement needs the spins");
   uint32_t* par = sm.par;
   uint32_t* sdraw = sm.sdraw;
@@ -200,49 +219,69 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
   // global memory only after the preceding kernel of the sweep is done
   pdl_wait();
 
-  // ---- phase 1: bonds, runs and draws of this thread's row word
-  const int r = threadIdx.x;
+  // ---- phase 1: bonds, runs and draws of this thread's row word; with K > 1
+  // the word's tasks (a bond direction each, then the draws) are dealt to its
+  // K threads, which lie in different warps
+  const int r = threadIdx.x & (ROWS - 1), part = K == 1 ? 0 : (int)threadIdx.x / ROWS;
+  static_assert((ROWS & (ROWS - 1)) == 0, "rows by mask");
   const int ry = r % TY, rz = r / TY;
   const int y = tc.y0 + ry, z = tc.z0 + rz;
   const bool rowv = (y < L) && (D == 2 || z < L);
   const int y1 = (y + 1 == L) ? 0 : y + 1;
   const int z1 = (D == 3) ? ((z + 1 == L) ? 0 : z + 1) : 0;
-  uint32_t X = 0u, Y = 0u, Z = 0u, S = 0u, XW = 0u;
+  const bool in_y = y1 - tc.y0 >= 0 && y1 - tc.y0 < TY, in_z = D == 3 && z1 - tc.z0 >= 0 && z1 - tc.z0 < TZ;
+  auto task = [&](int t) { return K == 1 || t % K == part; };
+  uint32_t A0 = 0u, A1 = 0u, A2 = 0u;
   if (rowv) {
     const uint32_t row = (uint32_t)y + (uint32_t)L * (uint32_t)z;
-    sm.srow[r] = row * (uint32_t)L + (uint32_t)tc.x0;
+    if (task(0)) sm.srow[r] = row * (uint32_t)L + (uint32_t)tc.x0;
     const uint32_t g = row * (uint32_t)lat.W + (uint32_t)tc.tx;
-    uint32_t A0, A1, A2 = 0u;
     if (FROM_MASK) {
-      A0 = __ldg(&lat.planes[g]) & vmask;
-      A1 = __ldg(&lat.planes[plane + g]) & vmask;
-      if (D == 3) A2 = __ldg(&lat.planes[2 * plane + g]) & vmask;
+      if (task(0)) A0 = __ldg(&lat.planes[g]) & vmask;
+      if (task(1)) A1 = __ldg(&lat.planes[plane + g]) & vmask;
+      if (D == 3 && task(2)) A2 = __ldg(&lat.planes[2 * plane + g]) & vmask;
     } else {
-      RowBytes rb;
+      const uint8_t* s = static_cast<const uint8_t*>(lat.spins);
+      const bool vec16 = (L & 15) == 0;
+      const uint32_t rowL = row * (uint32_t)L;
       const uint32_t row_y = (uint32_t)y1 + (uint32_t)L * (uint32_t)z;
       const uint32_t row_z = (uint32_t)y + (uint32_t)L * (uint32_t)z1;
-      load_rows<D>(static_cast<const uint8_t*>(lat.spins), L, tc.x0, row, row_y, row_z, rb);
       // equality masks (and the measurement) first, so the row bytes are
       // dead before the Bernoulli words are drawn
-      const uint32_t e0 = eq_bits(rb.a, rb.ax) & vmask;
-      const uint32_t e1 = eq_bits(rb.a, rb.ay) & vmask;
-      const uint32_t e2 = (D == 3) ? (eq_bits(rb.a, rb.az) & vmask) : 0u;
-      if (MEASURE) measure_row<D, MM>(rb, e0, e1, e2, vmask, nvalid, lat.q, m_acc, e_acc, s_whist + warp * kSmallQ, s_hist);
-      A0 = e0 ? (e0 & bernoulli_word(g, sweep, 0, lat.t_bond, e0, lat.rk)) : 0u;
-      A1 = e1 ? (e1 & bernoulli_word(g, sweep, 1, lat.t_bond, e1, lat.rk)) : 0u;
-      if (D == 3) A2 = e2 ? (e2 & bernoulli_word(g, sweep, 2, lat.t_bond, e2, lat.rk)) : 0u;
-      lat.planes[g] = A0;
-      lat.planes[plane + g] = A1;
-      if (D == 3) lat.planes[2 * plane + g] = A2;
+      uint32_t e0 = 0u, e1 = 0u, e2 = 0u;
+      {
+        uint32_t w[9];
+        load32<true>(s, rowL + (uint32_t)tc.x0, vec16, w);
+        if (MEASURE && task(D)) measure_state<MM>(w, vmask, nvalid, lat.q, m_acc, s_whist + warp * kSmallQ, s_hist);
+        uint32_t n[8];
+        if (task(1)) {
+          load32<false>(s, row_y * (uint32_t)L + (uint32_t)tc.x0, vec16, n);
+          e1 = eq_bits(w, n) & vmask;
+        }
+        if (D == 3 && task(2)) {
+          load32<false>(s, row_z * (uint32_t)L + (uint32_t)tc.x0, vec16, n);
+          e2 = eq_bits(w, n) & vmask;
+        }
+        if (task(0)) {
+          shift_row(s, w, rowL, L, tc.x0, nvalid, n);
+          e0 = eq_bits(w, n) & vmask;
+        }
+      }
+      if (MEASURE) {
+        const int par_bonds = __popc(e0) + __popc(e1) + (D == 3 ? __popc(e2) : 0);
+        const int nbonds = (task(D) ? D : 0) * nvalid;  // counted once a row word
+        e_acc += MM == 1 ? nbonds - 2 * par_bonds : nbonds - par_bonds;
+      }
+      if (e0) A0 = e0 & bernoulli_word(g, sweep, 0, lat.t_bond, e0, lat.rk);
+      if (e1) A1 = e1 & bernoulli_word(g, sweep, 1, lat.t_bond, e1, lat.rk);
+      if (D == 3 && e2) A2 = e2 & bernoulli_word(g, sweep, 2, lat.t_bond, e2, lat.rk);
+      if (task(0)) lat.planes[g] = A0;
+      if (task(1)) lat.planes[plane + g] = A1;
+      if (D == 3 && task(2)) lat.planes[2 * plane + g] = A2;
     }
-    X = A0 & (vmask >> 1);          // x-bonds whose +x site is in the same word
-    S = ~(X << 1) & vmask;          // x-run starts
-    XW = (tc.x0 == 0 && L <= 32) ? ((A0 >> (L - 1)) & 1u) : 0u;  // wrap inside the word
-    Y = (y1 - tc.y0 >= 0 && y1 - tc.y0 < TY) ? A1 : 0u;
-    Z = (D == 3 && z1 - tc.z0 >= 0 && z1 - tc.z0 < TZ) ? A2 : 0u;
     if (draws && two_state) {
       // two-state cluster draws: bit (x & 31) of word 0 of Philox(g, sweep, DRAW, 1)
-      sdraw[r] = philox(g, sweep, kDraw, 1u, lat.rk).x;
+      if (task(D)) sdraw[r] = philox(g, sweep, kDraw, 1u, lat.rk).x;
     } else if (draws && Smem::kPottsDraws) {
       // Potts cluster draw of every site: word (i & 3) of Philox(i >> 2, sweep, DRAW, 0)
       const uint32_t i0 = row * (uint32_t)L + (uint32_t)tc.x0;
@@ -252,7 +291,7 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
         // word starts a Philox group, and group j holds the draws of its
         // sites 4j..4j+3 (those past the end of the row go unused)
 #pragma unroll 1
-        for (int j = 0; j < 8; ++j) {
+        for (int j = part; j < 8; j += K) {
           const uint4 w = philox((i0 >> 2) + (uint32_t)j, sweep, kDraw, 0u, lat.rk);
           sdraw[j * (ROWS + 1) + r] = draw_value(w.x, dq) | (draw_value(w.y, dq) << 8) |
                                       (draw_value(w.z, dq) << 16) | (draw_value(w.w, dq) << 24);
@@ -261,7 +300,7 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
         uint32_t cached = 0xffffffffu;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
-        for (int j = 0; j < 8; ++j) {
+        for (int j = part * (8 / K); j < (part + 1) * (8 / K); ++j) {
           uint32_t packed = 0u;
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
@@ -280,28 +319,40 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
       }
     }
   }
-  sX[r] = X;
-  sY[r] = Y;
-  if (D == 3) sm.sZ[r] = Z;
+  // x-bonds whose +x site is in the same word (and, for a one-word row, the
+  // bond around it in bit 31: no bond inside the word has that bit), y- and
+  // z-bonds inside the tile
+  if (task(0)) {
+    const bool around = tc.x0 == 0 && L <= 32 && ((A0 >> (L - 1)) & 1u);
+    sX[r] = (A0 & (vmask >> 1)) | (around ? 0x80000000u : 0u);
+  }
+  if (task(1)) sY[r] = in_y ? A1 : 0u;
+  if (D == 3 && task(2)) sm.sZ[r] = in_z ? A2 : 0u;
   __syncthreads();
 
   // ---- phase 2a: the first bond of every x-run to the rows before it hooks
   // the run's start there (a plain store: each start is written by its own
   // row's thread only, and its new parent has a smaller index)
   const uint32_t cap = lat.cap;
-  uint32_t Y2 = 0u, Z2 = 0u, Sy = 0u, Sz = 0u;
+  uint32_t Y2 = 0u, Z2 = 0u, Sy = 0u, Sz = 0u, S = 0u, XW = 0u;
+  constexpr uint32_t kInWord = 0x7fffffffu;
+  // this thread's bits of the row word
+  const uint32_t own_bits = K == 1 ? kFull : ((1u << (32 / K % 32)) - 1u) << (32 / K * part);
   if (rowv) {
+    const uint32_t XX = sX[r], X = XX & kInWord;
+    S = ~(X << 1) & vmask;  // x-run starts
+    XW = XX >> 31;
     const uint32_t Yp = ry > 0 ? sY[r - 1] : 0u;
     const uint32_t Zp = (D == 3 && rz > 0) ? sm.sZ[r - TY] : 0u;
     const uint32_t joined = X << 1;  // bit b: site b is bonded to site b - 1
     uint32_t both = 0u;
     if (Yp) {
-      const uint32_t Xn = sX[r - 1];
+      const uint32_t Xn = sX[r - 1] & kInWord;
       Sy = ~(Xn << 1) & vmask;
       Y2 = Yp & ~((Yp & X & Xn) << 1);
     }
     if (D == 3 && Zp) {
-      const uint32_t Xn = sX[r - TY];
+      const uint32_t Xn = sX[r - TY] & kInWord;
       Sz = ~(Xn << 1) & vmask;
       Z2 = Zp & ~((Zp & X & Xn) << 1);
     }
@@ -312,7 +363,9 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
     uint32_t F = both & ~((((seed + joined) ^ joined) | seed) & joined);
     Z2 &= ~(F & ~Y2);
     const uint32_t FY = F & Y2;
-    Y2 &= ~F;
+    Y2 &= ~F & own_bits;
+    Z2 &= own_bits;
+    F &= own_bits;
     while (F) {
       const int b = __ffs(F) - 1;
       F &= F - 1u;
@@ -336,23 +389,23 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
              lat.err, cap);
     }
     // bonds around the torus inside the tile (a lattice no longer than it)
-    if (y1 < y && Y) {
+    if (y1 < y && in_y) {
       const int rn = r + (y1 - y);
       const uint32_t Sn = ~(sX[rn] << 1) & vmask;
-      for (uint32_t U = Y; U; U &= U - 1u) {
+      for (uint32_t U = sY[r] & own_bits; U; U &= U - 1u) {
         const int b = __ffs(U) - 1;
         sunion(par, (uint32_t)(32 * r) + run_start(S, b), (uint32_t)(32 * rn) + run_start(Sn, b), lat.err, cap);
       }
     }
-    if (D == 3 && z1 < z && Z) {
+    if (D == 3 && z1 < z && in_z) {
       const int rn = r + TY * (z1 - z);
       const uint32_t Sn = ~(sX[rn] << 1) & vmask;
-      for (uint32_t U = Z; U; U &= U - 1u) {
+      for (uint32_t U = sm.sZ[r] & own_bits; U; U &= U - 1u) {
         const int b = __ffs(U) - 1;
         sunion(par, (uint32_t)(32 * r) + run_start(S, b), (uint32_t)(32 * rn) + run_start(Sn, b), lat.err, cap);
       }
     }
-    if (XW) sunion(par, (uint32_t)(32 * r) + run_start(S, L - 1), (uint32_t)(32 * r), lat.err, cap);
+    if (XW && part == 0) sunion(par, (uint32_t)(32 * r) + run_start(S, L - 1), (uint32_t)(32 * r), lat.err, cap);
   }
   __syncthreads();
 
@@ -427,12 +480,16 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
   }
 }
 
-// Five 256-thread CTAs per SM, proportionally more of smaller tiles.
-template <int D, bool FROM_MASK, int MM>
-__global__ void __launch_bounds__(Tile<D>::THREADS, 5 * 256 / Tile<D>::THREADS)
+// Threads of an SM the split labeling counts on (64 registers a thread).
+constexpr int kLabelSplitThreads = 1024;
+
+// K threads per row word (label_split).  K = 1: five 256-thread CTAs per SM,
+// proportionally more of smaller tiles.
+template <int D, int K, bool FROM_MASK, int MM>
+__global__ void __launch_bounds__(K* Tile<D>::THREADS, K == 1 ? 5 * 256 / Tile<D>::THREADS : kLabelSplitThreads / (K * Tile<D>::THREADS))
     k_label(const __grid_constant__ Lattice lat, uint32_t sweep, const __grid_constant__ Measure mb) {
-  __shared__ LabelSmem<Tile<D>, MM> sm;
-  label_tile<Tile<D>, FROM_MASK, MM>(lat, blockIdx.x, sweep, mb, sm);
+  __shared__ LabelSmem<Tile<D>, MM, K> sm;
+  label_tile<Tile<D>, K, FROM_MASK, MM>(lat, blockIdx.x, sweep, mb, sm);
 }
 
 // Ising/Potts lattices of a batch, one tile of shape S per CTA; sweep
@@ -464,9 +521,9 @@ __device__ __forceinline__ void label_batch_entry(const BatchView& bv, uint32_t 
   if (step >= m.nsweeps) return;  // the member has had its sweeps this call
   const uint32_t sweep = m.sweep0 + step + 1u;
   const bool potts = LAYOUT == 2 || (LAYOUT == 3 && s_lat.model == kPotts);
-  if (step == 0u && !m.measure0) label_tile<S, false, 0>(s_lat, tile, sweep, m.meas, sm);
-  else if (LAYOUT != 1 && potts) label_tile<S, false, 2>(s_lat, tile, sweep, m.meas, sm);
-  else if (LAYOUT != 2) label_tile<S, false, 1>(s_lat, tile, sweep, m.meas, sm);
+  if (step == 0u && !m.measure0) label_tile<S, 1, false, 0>(s_lat, tile, sweep, m.meas, sm);
+  else if (LAYOUT != 1 && potts) label_tile<S, 1, false, 2>(s_lat, tile, sweep, m.meas, sm);
+  else if (LAYOUT != 2) label_tile<S, 1, false, 1>(s_lat, tile, sweep, m.meas, sm);
 }
 
 // PERSISTENT false: CTA k labels tile-map entry first + k (the grid covers
@@ -540,7 +597,7 @@ __global__ void __launch_bounds__(256) k_measure_rows(const __grid_constant__ La
     const uint32_t y1 = (y + 1u == (uint32_t)L) ? 0u : y + 1u;
     const uint32_t z1 = (D == 3) ? ((z + 1u == (uint32_t)L) ? 0u : z + 1u) : 0u;
     RowBytes rb;
-    load_rows<D>(static_cast<const uint8_t*>(lat.spins), L, x0, row, y1 + (uint32_t)L * z, y + (uint32_t)L * z1, rb);
+    load_rows<D>(static_cast<const uint8_t*>(lat.spins), L, x0, nvalid, row, y1 + (uint32_t)L * z, y + (uint32_t)L * z1, rb);
     const uint32_t e0 = eq_bits(rb.a, rb.ax) & vmask;
     const uint32_t e1 = eq_bits(rb.a, rb.ay) & vmask;
     const uint32_t e2 = (D == 3) ? (eq_bits(rb.a, rb.az) & vmask) : 0u;
@@ -825,17 +882,43 @@ void tiles_for(int dim, int L, int* ntx, int* nty, int* ntz, int shape) {
 }
 
 namespace {
+
+// Threads per row word of a lattice's labeling: the most (4, 2 or 1) with
+// which the GPU holds all tiles at once.  With few tiles the kernel is a chain
+// of latencies -- a thread's three Bernoulli words, its hooks and unions, its
+// rows' walks -- and the threads added shorten every link; once the tiles
+// come in waves the extra row-word arithmetic only costs.  us per sweep with
+// 1, 2 and 4 threads: 2D L = 128 27.9 / 22.5 / 20.4, 515 32.2 / 26.6 / 24.1,
+// 1024 (256 tiles) 31.1 / 27.7 / 27.4, 1448 (552) 36.7 / 33.9 / 38.9; 3D L =
+// 32 29.8 / 27.1 / 26.9, 100 (196 tiles of twice the size) 41.5 / 40.1 /
+// 43.2, 128 (256) 44.2 / 43.1 / 50.1, 161 (726) 68.9 / 71.7 / 84.3.
+template <int D>
+int label_split(const Lattice& lat) {
+  const int tiles = lat.ntx * lat.nty * lat.ntz;
+  const int whole = sm_count() * (kLabelSplitThreads / Tile<D>::THREADS);  // tiles held at K = 1
+  return 4 * tiles <= whole ? 4 : 2 * tiles <= whole ? 2 : 1;
+}
+
+template <int D, bool FROM_MASK, int MM>
+cudaError_t launch_label_kernel(const Lattice& lat, uint32_t sweep, const Measure& m, cudaStream_t st) {
+  const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz), t = (unsigned)Tile<D>::THREADS;
+  switch (label_split<D>(lat)) {
+    case 4: return launch_pdl(k_label<D, 4, FROM_MASK, MM>, g, 4 * t, st, lat, sweep, m);
+    case 2: return launch_pdl(k_label<D, 2, FROM_MASK, MM>, g, 2 * t, st, lat, sweep, m);
+    default: return launch_pdl(k_label<D, 1, FROM_MASK, MM>, g, t, st, lat, sweep, m);
+  }
+}
+
 template <int D>
 cudaError_t launch_label_dim(const Lattice& lat, uint32_t sweep, bool from_mask, bool potts_draws,
                              cudaStream_t st) {
-  const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz), t = (unsigned)Tile<D>::THREADS;
   const Measure none{};
   if (from_mask) {
-    if (potts_draws) return launch_pdl(k_label<D, true, 3>, g, t, st, lat, sweep, none);
-    return launch_pdl(k_label<D, true, 0>, g, t, st, lat, sweep, none);
+    if (potts_draws) return launch_label_kernel<D, true, 3>(lat, sweep, none, st);
+    return launch_label_kernel<D, true, 0>(lat, sweep, none, st);
   }
-  if (potts_draws) return launch_pdl(k_label<D, false, 3>, g, t, st, lat, sweep, none);
-  return launch_pdl(k_label<D, false, 0>, g, t, st, lat, sweep, none);
+  if (potts_draws) return launch_label_kernel<D, false, 3>(lat, sweep, none, st);
+  return launch_label_kernel<D, false, 0>(lat, sweep, none, st);
 }
 }  // namespace
 
@@ -907,17 +990,12 @@ cudaError_t launch_measure_rows(const Lattice& lat, uint32_t sweep, const Measur
 
 cudaError_t launch_label_measured(const Lattice& lat, uint32_t sweep, const Measure& m,
                                   cudaStream_t st) {
-  const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz);
-  cudaError_t e = cudaSuccess;
   const bool potts = lat.model == kPotts;
-  if (lat.dim == 2) {
-    if (potts) e = launch_pdl(k_label<2, false, 2>, g, (unsigned)Tile<2>::THREADS, st, lat, sweep, m);
-    else e = launch_pdl(k_label<2, false, 1>, g, (unsigned)Tile<2>::THREADS, st, lat, sweep, m);
-  } else {
-    if (potts) e = launch_pdl(k_label<3, false, 2>, g, (unsigned)Tile<3>::THREADS, st, lat, sweep, m);
-    else e = launch_pdl(k_label<3, false, 1>, g, (unsigned)Tile<3>::THREADS, st, lat, sweep, m);
-  }
-  return e;
+  if (lat.dim == 2)
+    return potts ? launch_label_kernel<2, false, 2>(lat, sweep, m, st)
+                 : launch_label_kernel<2, false, 1>(lat, sweep, m, st);
+  return potts ? launch_label_kernel<3, false, 2>(lat, sweep, m, st)
+               : launch_label_kernel<3, false, 1>(lat, sweep, m, st);
 }
 
 cudaError_t launch_bonds_xy(const Lattice& lat, uint32_t sweep, const Measure* m, int* blocks,

@@ -94,3 +94,30 @@ def test_small_members_over_several_launches(sw):
         sw.sw_batch_destroy(b)
         for h in hs:
             sw.sw_destroy(h)
+
+
+@pytest.mark.parametrize("model,dim,L,q", [
+    # four threads a row word: rows at every alignment, whole and half words
+    (ISING, 2, 113, 2), (ISING, 2, 114, 2), (POTTS, 2, 115, 5), (ISING, 2, 144, 2), (POTTS, 2, 176, 17),
+    (ISING, 3, 23, 2), (POTTS, 3, 26, 4), (ISING, 3, 48, 2),
+    # two
+    (POTTS, 2, 1185, 3), (ISING, 3, 99, 2), (POTTS, 3, 100, 3),
+    # one
+    (ISING, 2, 1801, 2), (POTTS, 3, 161, 3)])
+def test_tiled_sweeps_split_and_ragged(sw, model, dim, L, q):
+    T = 2.27 if model == ISING and dim == 2 else 4.5 if model == ISING else 0.95 if dim == 2 else 1.8
+    h = sw.sw_create(model, dim, L, q, T, 5 + L)
+    o = oracle.Oracle(model, dim, L, q, T, 5 + L)
+    try:
+        sw.sw_sweep(h, 2)
+        sw.sw_discard(h, 1)
+        o.sweep(2)
+        o.sweep(1, measure=False)
+        assert np.array_equal(sw.sw_get_bonds(h), o.planes)
+        assert np.array_equal(sw.sw_get_labels(h), o.labels)
+        assert np.array_equal(sw.sw_get_spins(h), o.spins)
+        got, ref = sw.sw_measure(h), o.take_acc()
+        assert all(got[f] == ref[f] for f in ref)
+    finally:
+        sw.sw_destroy(h)
+        o.close()
