@@ -623,6 +623,17 @@ __global__ void __launch_bounds__(256) k_measure_rows(const __grid_constant__ La
 }
 
 // ---------------------------------------------------------------- XY bonds
+// 1 + the top 23 bits of w as a fraction (a bit pattern: no conversion, which
+// would share the exp's pipe).
+__device__ __forceinline__ float unit_bits(uint32_t w) { return __uint_as_float(0x3f800000u | (w >> 9)); }
+
+// 2^x, within 2^-22 relative (the hardware approximation).
+__device__ __forceinline__ float fast_exp2(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // One CTA per 32 x BY (x BZ) block of sites, grid-strided over the blocks.
 // The projections (x, y) = (cos, sin)(theta - phi) on the sweep's mirror
 // axis are computed once per site of the block and its +x/+y/+z halo into
@@ -645,12 +656,27 @@ struct XYBlock<3> {
   static constexpr int BY = 16, BZ = 8;
 };
 
+//
+// The kernel is issue-bound (65% of issue slots): a lane's Philox word and its
+// sincosf are about half of its instructions, so the rest was cut -- the bond
+// decision without an integer conversion, a warp's row coordinates by
+// constants, and its bond words kept a lane per row and stored once per block
+// instead of a predicated store per row and direction.  3D L = 256: 145.1 M ->
+// 117.0 M warp instructions, 183.1 -> 150.6 us measured, 173.8 -> 139.9 not;
+// the sweep 307 -> 273 us.
+//
+// CTAs per SM of the one-wave grid.  Fixed, not asked of the occupancy
+// calculator: the partial sums of the measurement are added in an order that
+// depends on the grid.
+constexpr int kXYBlocksPerSM[2] = {6, 5};
+
 template <int D, bool MEASURE>
-__global__ void __launch_bounds__(256) k_bonds_xy(const __grid_constant__ Lattice lat, uint32_t sweep,
-                                                   const __grid_constant__ Measure mb) {
+__global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
+    k_bonds_xy(const __grid_constant__ Lattice lat, uint32_t sweep, const __grid_constant__ Measure mb) {
   constexpr int BY = XYBlock<D>::BY, BZ = XYBlock<D>::BZ;
   constexpr int HX = 33, HY = BY + 1, HZ = (D == 3) ? BZ + 1 : 1, NBOX = HX * HY * HZ;
-  constexpr int NW = 256 / 32;
+  constexpr int NW = 256 / 32, RW = BY * BZ / NW;  // rows per warp
+  static_assert(BY % NW == 0 && RW <= 32 && HY >= NW, "a lane per row of the warp");
   __shared__ float2 sv[NBOX];
   __shared__ float s_phi;
   __shared__ double s_rd[NW];
@@ -658,6 +684,7 @@ __global__ void __launch_bounds__(256) k_bonds_xy(const __grid_constant__ Lattic
   pdl_wait();
   __syncthreads();
   const float phi = s_phi;
+  const float kexp = -__fmul_rn(lat.twoK, 0x1.715476p+0f);  // -2K log2 e
   const int L = lat.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t plane = lat.R * (uint32_t)lat.W;
   const float* th = static_cast<const float*>(lat.spins);
@@ -669,44 +696,48 @@ __global__ void __launch_bounds__(256) k_bonds_xy(const __grid_constant__ Lattic
     const int x0 = 32 * (int)(t % nbx), y0 = BY * (int)((t / nbx) % nby), z0 = BZ * (int)(t / (nbx * nby));
     const int nx = min(32, L - x0), ny = min(BY, L - y0), nz = (D == 3) ? min(BZ, L - z0) : 1;
     __syncthreads();  // the previous block's values are no longer read
-    // a warp per halo row (yy, zz), lanes along x; then the +x halo column
-    // (entry 32 of every row) a thread per row
-    for (int hr = warp; hr < HY * HZ; hr += NW) {
-      const int yy = hr % HY, zz = hr / HY;
-      if (yy > ny || zz > nz || lane > nx) continue;  // beyond the valid sites and their halo
-      int gy = y0 + yy, gz = (D == 3) ? z0 + zz : 0;
-      if (gy >= L) gy -= L;
-      if (gz >= L) gz -= L;
-      int gx = x0 + lane;
+    auto project = [&](int yy, int zz, int xx) {
+      int gx = x0 + xx, gy = y0 + yy, gz = (D == 3) ? z0 + zz : 0;
       if (gx >= L) gx -= L;
+      if (gy >= L) gy -= L;
+      if (D == 3 && gz >= L) gz -= L;
       float sn, cs;
       sincosf(__fsub_rn(__ldg(&th[(uint32_t)gx + (uint32_t)L * ((uint32_t)gy + (uint32_t)L * (uint32_t)gz)]),
                         phi), &sn, &cs);
-      sv[hr * HX + lane] = make_float2(cs, sn);
-    }
-    if (nx == 32) {
+      sv[(yy + HY * zz) * HX + xx] = make_float2(cs, sn);
+    };
+    // a warp per halo row (yy, zz), lanes along x; then the +x halo column
+    // (entry 32 of every row) a thread per row
+    if (lane <= nx)
+      for (int yy = warp, zz = 0; zz < HZ && zz <= nz;) {
+        if (yy <= ny) project(yy, zz, lane);
+        yy += NW;
+        if (yy >= HY) {
+          yy -= HY;
+          ++zz;
+        }
+      }
+    if (nx == 32)
       for (int hr = threadIdx.x; hr < HY * HZ; hr += 256) {
         const int yy = hr % HY, zz = hr / HY;
-        if (yy > ny || zz > nz) continue;
-        int gy = y0 + yy, gz = (D == 3) ? z0 + zz : 0;
-        if (gy >= L) gy -= L;
-        if (gz >= L) gz -= L;
-        int gx = x0 + 32;
-        if (gx >= L) gx -= L;
-        float sn, cs;
-        sincosf(__fsub_rn(__ldg(&th[(uint32_t)gx + (uint32_t)L * ((uint32_t)gy + (uint32_t)L * (uint32_t)gz)]),
-                          phi), &sn, &cs);
-        sv[hr * HX + 32] = make_float2(cs, sn);
+        if (yy <= ny && zz <= nz) project(yy, zz, 32);
       }
-    }
     __syncthreads();
-    for (int rr = warp; rr < BY * BZ; rr += NW) {
-      const int yy = rr % BY, zz = rr / BY;
-      const bool rowv = yy < ny && zz < nz;
-      uint32_t a = 0u;
-      if (rowv && lane < nx) {
-        const uint32_t y = (uint32_t)(y0 + yy), z = (uint32_t)(z0 + zz);
-        const uint32_t i = (uint32_t)(x0 + lane) + (uint32_t)L * (y + (uint32_t)L * z);
+    // a warp's rows in turn, row k = (warp + 8 (k mod BY / 8), k / (BY / 8));
+    // lane k keeps row k's bond words
+    uint32_t m[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) m[d] = 0u;
+    const uint32_t i0 = (uint32_t)(x0 + lane) + (uint32_t)L * ((uint32_t)(y0 + warp) + (uint32_t)L * (uint32_t)z0);
+    constexpr int RY = BY / NW;  // rows of the warp per z
+#pragma unroll 2
+    for (int k = 0; k < RW; ++k) {
+      const int yy = warp + NW * (k % RY), zz = k / RY;
+      bool act[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) act[d] = false;
+      if (yy < ny && zz < nz && lane < nx) {
+        const uint32_t i = i0 + (uint32_t)L * ((uint32_t)(NW * (k % RY)) + (uint32_t)L * (uint32_t)zz);
         const uint4 w = philox(i, sweep, kBond, 0u, lat.rk);
         const int c = lane + HX * (yy + HY * zz);
         const float2 si = sv[c];
@@ -714,18 +745,17 @@ __global__ void __launch_bounds__(256) k_bonds_xy(const __grid_constant__ Lattic
         for (int d = 0; d < D; ++d) {
           const float2 sj = sv[c + (d == 0 ? 1 : d == 1 ? HX : HX * HY)];
           const float prod = __fmul_rn(si.x, sj.x);
-          bool act = false;
-          if (prod > 0.0f) {
-            // u < p with p = -expm1f(-2K prod): a fast estimate of p decides
-            // unless u lies within a margin far above the estimate's error
-            // (|a| <= 2K keeps __expf within a few ulp), where expm1f decides
-            const float a2 = __fmul_rn(lat.twoK, prod);
+          // u < p with p = -expm1f(-2K prod), u = (w >> 8) 2^-24: the sign
+          // of (1 + u) + exp(-2K prod) - 2 decides, with u cut to 23 bits
+          // and a fast exp, unless it lies within a margin far above their
+          // error (2^-23 and a few ulp), where expm1f decides
+          const float near = __fsub_rn(
+              __fadd_rn(unit_bits(word_of(w, d)), fast_exp2(__fmul_rn(kexp, prod))), 2.0f);
+          act[d] = prod > 0.0f && near < 0.0f;
+          if (prod > 0.0f && fabsf(near) <= 0x1p-16f) {
             const float u = __fmul_rn((float)(word_of(w, d) >> 8), 0x1p-24f);
-            const float pf = __fsub_rn(1.0f, __expf(-a2));
-            if (fabsf(__fsub_rn(u, pf)) > 0x1p-16f) act = u < pf;
-            else act = u < -expm1f(-a2);
+            act[d] = u < -expm1f(-__fmul_rn(lat.twoK, prod));
           }
-          a |= (uint32_t)act << d;
           if (MEASURE) fe = __fadd_rn(fe, __fadd_rn(prod, __fmul_rn(si.y, sj.y)));
         }
         if (MEASURE) {
@@ -733,11 +763,18 @@ __global__ void __launch_bounds__(256) k_bonds_xy(const __grid_constant__ Lattic
           fy = __fadd_rn(fy, si.y);
         }
       }
-      const uint32_t row = (uint32_t)(y0 + yy) + (uint32_t)L * (uint32_t)(z0 + zz);
 #pragma unroll
       for (int d = 0; d < D; ++d) {
-        const uint32_t bal = __ballot_sync(kFull, (a >> d) & 1u);
-        if (rowv && lane == d) lat.planes[d * plane + row * (uint32_t)lat.W + (uint32_t)(x0 >> 5)] = bal;
+        const uint32_t bal = __ballot_sync(kFull, act[d]);
+        if (lane == k) m[d] = bal;
+      }
+    }
+    {
+      const int yy = warp + NW * (lane % RY), zz = lane / RY;
+      if (lane < RW && yy < ny && zz < nz) {
+        const uint32_t g = ((uint32_t)(y0 + yy) + (uint32_t)L * (uint32_t)(z0 + zz)) * (uint32_t)lat.W + (uint32_t)(x0 >> 5);
+#pragma unroll
+        for (int d = 0; d < D; ++d) lat.planes[d * plane + g] = m[d];
       }
     }
   }
@@ -787,6 +824,7 @@ __global__ void __launch_bounds__(256) k_bonds_clock(const __grid_constant__ Lat
   // the draw rounded to float): below 2K * 2.5e-7 + 4e-7; the margin is
   // about four times that, and draws inside it read the exact entry.
   const float margin = __fadd_rn(0x1p-16f, __fmul_rn(lat.twoK, 0x1p-20f));
+  const float kexp = -__fmul_rn(lat.twoK, 0x1.715476p+0f);  // -2K log2 e
   const int mirror = (int)s_mirror;
   const uint32_t nwords = lat.R * (uint32_t)lat.W;
   const uint32_t plane = nwords;
@@ -837,9 +875,8 @@ __global__ void __launch_bounds__(256) k_bonds_clock(const __grid_constant__ Lat
         bool act = false;
         if (prod > 0.0f) {
           const uint32_t wd = word_of(w, d);
-          const float pf = __fsub_rn(1.0f, __expf(-__fmul_rn(lat.twoK, prod)));
-          const float diff = __fsub_rn(__fmul_rn(__uint2float_rn(wd), 0x1p-32f), pf);
-          act = (fabsf(diff) > margin) ? diff < 0.0f
+          const float near = __fsub_rn(__fadd_rn(unit_bits(wd), fast_exp2(__fmul_rn(kexp, prod))), 2.0f);
+          act = (fabsf(near) > margin) ? near < 0.0f
                                        : wd < __ldg(&lat.ctab[(size_t)ki * (size_t)q2 + (size_t)kj]);
         }
         a |= (uint32_t)act << d;
@@ -1004,12 +1041,12 @@ cudaError_t launch_bonds_xy(const Lattice& lat, uint32_t sweep, const Measure* m
   const uint32_t nb = (lat.dim == 2)
                           ? (uint32_t)lat.W * (uint32_t)((lat.L + XYBlock<2>::BY - 1) / XYBlock<2>::BY)
                           : (uint32_t)lat.W * ny * (uint32_t)((lat.L + XYBlock<3>::BZ - 1) / XYBlock<3>::BZ);
-  // one wave: the CTAs the GPU holds at once (the box of projections and the
-  // registers allow five per SM), each striding over the blocks; at most
-  // kMeasureBlocks (the slots of the XY partials)
+  // one wave: the CTAs the GPU holds at once, each striding over the blocks;
+  // at most kMeasureBlocks (the slots of the XY partials)
   unsigned g = 0;
   auto launch = [&](auto kernel, const Measure& mm) {
-    g = batch_grid(kernel, 256, nb);
+    g = (unsigned)(sm_count() * kXYBlocksPerSM[lat.dim - 2]);
+    if (g > nb) g = nb;
     if (g > (unsigned)kMeasureBlocks) g = (unsigned)kMeasureBlocks;
     return launch_pdl(kernel, g, 256, st, lat, sweep, mm);
   };
