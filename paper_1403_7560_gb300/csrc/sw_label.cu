@@ -439,6 +439,10 @@ __device__ __forceinline__ void label_tile(const Lattice& lat, uint32_t tile, ui
           p[j] = up;
         }
       }
+      // the starts now point at their roots: rows are taken in rising order
+      // and parents lie in earlier rows, so later walks are short (3D L = 256:
+      // 70.8 M -> 67.3 M warp instructions, 88.5 -> 85.4 us)
+      *reinterpret_cast<uint4*>(par + t0) = make_uint4(p[0], p[1], p[2], p[3]);
       const uint32_t dr = !draws ? 0u
                           : (two_state || !Smem::kPottsDraws) ? sdraw[rr] >> b0
                                                               : sdraw[(lane & 7) * (ROWS + 1) + rr];
