@@ -203,7 +203,7 @@ int check_device_error(sw_handle* h) {
 // the labeling kernel, which also measures the incoming state when the
 // previous sweep's record is pending; XY and clock bonds come from their own
 // kernels, which measure the pending state the same way.  Sets *finalize to
-// the pending sweep whose record the flip kernel of this sweep must write
+// the pending sweep whose record this sweep's merge or flip must write
 // (0 if none).
 cudaError_t launch_bonds_labels(sw_handle* h, uint32_t k, uint32_t* finalize) {
   *finalize = 0u;
@@ -262,7 +262,7 @@ cudaError_t one_sweep(sw_handle* h, uint32_t k, bool measure, cudaEvent_t* ev) {
   if (ev) e = cudaEventRecord(ev[0], h->stream);
   if (e == cudaSuccess) e = launch_bonds_labels(h, k, &finalize);
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], h->stream);
-  if (e == cudaSuccess) e = swgb::launch_merge(h->lat, h->stream);
+  if (e == cudaSuccess) e = swgb::launch_merge(h->lat, h->meas, finalize, h->stream);
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], h->stream);
   // the flip writes the spins: a download of them goes first
   if (e == cudaSuccess) e = swgb::guard_state_write(h, h->lat.spins, h->stream);

@@ -28,11 +28,11 @@ namespace {
 
 using namespace dev;
 
-template <class S>
+template <class S, int K = 1>
 struct MergeShape {
   // face bonds a tile owns: +x face, +y face (and +z face)
   static constexpr int kMax = S::ROWS + 32 * S::TZ + (S::D == 3 ? 32 * S::TY : 0);
-  static constexpr int kPerThread = (kMax + S::THREADS - 1) / S::THREADS;
+  static constexpr int kPerThread = (kMax + K * S::THREADS - 1) / (K * S::THREADS);
 };
 
 template <class S>
@@ -44,11 +44,11 @@ struct MergeSmem {
 // faces: which of the tile's +x (1), +y (2), +z (4) faces to join; a merge
 // split into one launch per axis starts the tile's hooked list with the x
 // faces and appends to it in the later launches.
-template <class S>
+template <class S, int K = 1>
 __device__ __forceinline__ void merge_tile(const Lattice& lat, uint32_t tile, MergeSmem<S>& sm,
                                            uint32_t faces = 7u) {
-  constexpr int D = S::D, TY = S::TY, TZ = S::TZ, NT = S::THREADS;
-  constexpr int NC = MergeShape<S>::kPerThread;
+  constexpr int D = S::D, TY = S::TY, TZ = S::TZ, NT = K * S::THREADS;
+  constexpr int NC = MergeShape<S, K>::kPerThread;
   uint2* s_list = sm.list;
   int& s_n = sm.n;
   const TileCoord tc = tile_coord<S>(lat, tile);
@@ -126,11 +126,33 @@ __device__ __forceinline__ void merge_tile(const Lattice& lat, uint32_t tile, Me
 // Eight 256-thread CTAs per SM, proportionally more of smaller tiles.
 constexpr int merge_blocks(int threads) { return 8 * 256 / threads > 32 ? 32 : 8 * 256 / threads; }
 
-template <int D>
-__global__ void __launch_bounds__(Tile<D>::THREADS, merge_blocks(Tile<D>::THREADS))
-    k_merge(Lattice lat, uint32_t faces) {
+// Writes the record of sweep `finalize` by one whole CTA; out of line, so
+// that the kernel around it keeps its registers.
+template <int NW>
+__device__ __noinline__ void finalize_by_cta(const Lattice& lat, const Measure& mb, uint32_t finalize) {
+  __shared__ long long s_red[NW];
+  __shared__ double s_rd[NW];
+  finalize_record<NW>(lat, mb, finalize, s_red, s_rd);
+}
+
+// A CTA per tile, K threads a row word as in the labeling (tile_split: with
+// few tiles the merge is a chain of face loads and walks, and the threads added
+// take a tile's unions in fewer rounds; us per sweep with 1 / K threads: 3D
+// Ising L = 64 27.6 / 24.3, 100 35.9 / 33.3, 128 42.1 / 39.4).
+// With finalize != 0 the first CTA writes
+// the record of sweep `finalize` from the sums that this sweep's labeling left
+// (a chain of about 6 us that runs beside the merge; block 0 of the
+// compression held that kernel up with it).
+template <int D, int K>
+__global__ void __launch_bounds__(K* Tile<D>::THREADS, merge_blocks(K* Tile<D>::THREADS))
+    k_merge(const __grid_constant__ Lattice lat, const __grid_constant__ Measure mb, uint32_t finalize) {
+  if (finalize != 0u && blockIdx.x == 0u) {
+    pdl_wait();
+    finalize_by_cta<K * Tile<D>::THREADS / 32>(lat, mb, finalize);
+    return;
+  }
   __shared__ MergeSmem<Tile<D>> sm;
-  merge_tile<Tile<D>>(lat, blockIdx.x, sm, faces);
+  merge_tile<Tile<D>, K>(lat, blockIdx.x - (finalize != 0u ? 1u : 0u), sm);
 }
 
 // Batch kernels: PERSISTENT false launches one CTA per tile-map entry
@@ -160,6 +182,14 @@ __global__ void __launch_bounds__(S::THREADS, PERSISTENT ? (merge_blocks(S::THRE
 }
 
 constexpr int kFlipThreads = 256, kFlipWarps = kFlipThreads / 32;
+// Lattices up to this size are flipped without a compression: every site
+// walks from its tile's root to its cluster's (walk_roots).  The walks of a
+// small lattice are cheaper than one more launch of dependent walks; those of
+// a large one repeat too much.  us per sweep, walk / compression: 2D L = 160
+// 16.1 / 18.2, 1024 25.4 / 26.5, 2048 50.6 / 44.2; 3D Ising L = 32 21.4 /
+// 23.4, 100 36.1 / 39.0, 128 41.6 / 42.8, 160 59.9 / 57.3; clock L = 128 64.8
+// / 63.0.
+constexpr uint32_t kFlipWalkSites = 1u << 20;
 constexpr unsigned kFlipBlocks = 152u * 8u;
 
 // The roots one tile's merge hooked walk to their global root and store
@@ -191,13 +221,9 @@ __device__ __forceinline__ void compress_tile(const Lattice& lat, uint32_t t) {
 // Every root the merge hooked under another tree (the tiles' hooked lists)
 // walks to its global root and stores (root, marker, root draw) in its own
 // word, so that every site is at most two loads away from its cluster's
-// draw.  Block 0 first writes the record of the previous measured sweep,
-// from the sums its successor's labeling kernel left behind.
-__global__ void __launch_bounds__(kFlipThreads, 8) k_compress(Lattice lat, Measure mb, uint32_t finalize) {
-  __shared__ long long s_red[kFlipWarps];
-  __shared__ double s_rd[kFlipWarps];
+// draw.
+__global__ void __launch_bounds__(kFlipThreads, 8) k_compress(Lattice lat) {
   pdl_wait();
-  if (finalize != 0u && blockIdx.x == 0) finalize_record<kFlipWarps>(lat, mb, finalize, s_red, s_rd);
   const uint32_t ntiles = (uint32_t)(lat.ntx * lat.nty * lat.ntz);
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) compress_tile(lat, t);
 }
@@ -226,6 +252,37 @@ __global__ void __launch_bounds__(kFlipThreads, PERSISTENT ? 4 : 6) k_compress_b
   }
 }
 
+// The words of four consecutive sites' cluster roots, from their own words:
+// the walks take each step together (the forest is read-only here; L1 serves
+// the nodes that a warp's walks share).  Returns how many are roots.
+__device__ __forceinline__ int walk_roots(const Lattice& lat, uint32_t i0, uint32_t* v) {
+  const int shift = lat.sbits + 1;
+  uint32_t at[4], moved = 0u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    at[j] = i0 + (uint32_t)j;
+    moved |= (v[j] >> shift) ^ at[j];
+  }
+  uint32_t it = 0;
+  for (; it < lat.cap && moved; ++it) {
+    moved = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t up = v[j] >> shift;
+      if (up != at[j]) {
+        at[j] = up;
+        v[j] = __ldg(&lat.forest[up]);
+        moved |= (v[j] >> shift) ^ up;
+      }
+    }
+  }
+  if (moved) atomicExch(lat.err, kErrTimeout);
+  int roots = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) roots += at[j] == i0 + (uint32_t)j;
+  return roots;
+}
+
 // Every site takes its cluster's draw from its own word (local roots, now
 // compressed) or its local root's word and gets its new state: Ising and
 // Potts take the draw (Ising: 1 = -1); XY and clock reflect a drawn cluster
@@ -237,9 +294,20 @@ __global__ void __launch_bounds__(kFlipThreads, PERSISTENT ? 4 : 6) k_compress_b
 // lines, and L1 serves the repeats (the forest is read-only in this kernel).
 // All buffers come from the device pool, so these accesses are aligned; the
 // last N mod 4 sites are taken one by one.
-template <int MODEL>
+// WALK: no compression has run, and the four sites walk together from their
+// local roots to the cluster's root (walk_roots).
+// FINALIZE: the first CTA writes the previous record, beside the others (a
+// one-tile lattice has no merge to do it; an instantiation of its own, since
+// the call in the others' code cost them a third of their resident warps).
+template <int MODEL, bool WALK, bool FINALIZE = false>
 __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sweep, Measure mb,
-                                                         bool count) {
+                                                         bool count, uint32_t finalize) {
+  if (FINALIZE && blockIdx.x == 0u) {
+    pdl_wait();
+    finalize_by_cta<kFlipWarps>(lat, mb, finalize);
+    return;
+  }
+  const uint32_t block = blockIdx.x - (FINALIZE ? 1u : 0u), nblocks = gridDim.x - (FINALIZE ? 1u : 0u);
   __shared__ float s_phi;
   __shared__ uint32_t s_mirror;
   __shared__ long long s_red[kFlipWarps];
@@ -269,7 +337,7 @@ __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sw
     return __float_as_uint(t);
   };
   long long roots = 0;
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
+  for (uint32_t q = block * blockDim.x + threadIdx.x; q < nq; q += nblocks * blockDim.x) {
     const uint4 w4 = __ldcg(&f4[q]);
     uint32_t v[4] = {w4.x, w4.y, w4.z, w4.w};
     // XY and clock: the old states are loaded beside the forest words
@@ -284,9 +352,11 @@ __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sw
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+      if (WALK) continue;
       if (!(v[j] & lr_bit)) v[j] = __ldg(&lat.forest[v[j] >> shift]);
       else if ((v[j] >> shift) == 4u * q + (uint32_t)j) ++roots;  // a cluster's root
     }
+    if (WALK) roots += walk_roots(lat, 4u * q, v);
     uint32_t n[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) n[j] = update(old[j], v[j] & dmask);
@@ -298,14 +368,26 @@ __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sw
       static_cast<uint32_t*>(lat.spins)[q] = n[0] | (n[1] << 8) | (n[2] << 16) | (n[3] << 24);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x < (lat.N & 3u)) {
+  if (block == 0u && threadIdx.x < (lat.N & 3u)) {
     const uint32_t i = 4u * nq + threadIdx.x;
     uint32_t v = __ldcg(&lat.forest[i]);
     uint32_t old = 0u;
     if (MODEL == kXY) old = __ldcg(&static_cast<const uint32_t*>(lat.spins)[i]);
     if (MODEL == kClock) old = __ldcg(&static_cast<const uint16_t*>(lat.spins)[i]);
-    if (!(v & lr_bit)) v = __ldg(&lat.forest[v >> shift]);
-    else if ((v >> shift) == i) ++roots;
+    if (WALK) {
+      uint32_t at = i;
+      uint32_t it = 0;
+      for (; it < lat.cap && (v >> shift) != at; ++it) {
+        at = v >> shift;
+        v = __ldg(&lat.forest[at]);
+      }
+      if (it == lat.cap && (v >> shift) != at) atomicExch(lat.err, kErrTimeout);
+      roots += at == i;
+    } else if (!(v & lr_bit)) {
+      v = __ldg(&lat.forest[v >> shift]);
+    } else if ((v >> shift) == i) {
+      ++roots;
+    }
     const uint32_t n = update(old, v & dmask);
     if (MODEL == kXY) static_cast<uint32_t*>(lat.spins)[i] = n;
     else if (MODEL == kClock) static_cast<uint16_t*>(lat.spins)[i] = (uint16_t)n;
@@ -314,7 +396,7 @@ __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sw
   if (count) {
     const long long tot = block_combine<kFlipWarps>(warp_sum(roots), s_red);
     if (threadIdx.x == 0 && tot)
-      atomicAdd(mb.nclusters + kSlots * (sweep & 1u) + (blockIdx.x % kSlots), (unsigned long long)tot);
+      atomicAdd(mb.nclusters + kSlots * (sweep & 1u) + (block % kSlots), (unsigned long long)tot);
   }
 }
 
@@ -437,25 +519,62 @@ void tile_buffers(int model, int dim, int L, size_t* ntiles, size_t* hook_words)
   }
 }
 
-cudaError_t launch_merge(const Lattice& lat, cudaStream_t st) {
-  const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz);
-  if (lat.dim == 2) return launch_pdl(k_merge<2>, g, (unsigned)Tile<2>::THREADS, st, lat, 7u);
-  return launch_pdl(k_merge<3>, g, (unsigned)Tile<3>::THREADS, st, lat, 7u);
-}
+namespace {
 
-cudaError_t launch_flip(const Lattice& lat, int model, uint32_t sweep, const Measure& m, bool count,
-                        uint32_t finalize, cudaStream_t st) {
+bool flip_walks(const Lattice& lat) { return lat.N <= kFlipWalkSites; }
+// No bond leaves the tile of a one-tile lattice: nothing to merge.
+bool one_tile(const Lattice& lat) { return lat.ntx * lat.nty * lat.ntz == 1; }
+
+template <int MODEL>
+cudaError_t launch_apply(const Lattice& lat, uint32_t sweep, const Measure& m, bool count, uint32_t finalize,
+                         cudaStream_t st) {
   // a thread per four sites; at most kFlipBlocks CTAs striding over them
   unsigned g = (unsigned)((lat.N + 4u * kFlipThreads - 1) / (4u * kFlipThreads));
   if (g > kFlipBlocks) g = kFlipBlocks;
   if (g == 0) g = 1;
-  const unsigned ntiles = (unsigned)(lat.ntx * lat.nty * lat.ntz);
-  const cudaError_t e = launch_pdl(k_compress, ntiles, kFlipThreads, st, lat, m, finalize);
-  if (e != cudaSuccess) return e;
-  if (model == kIsing) return launch_pdl(k_apply<kIsing>, g, kFlipThreads, st, lat, sweep, m, count);
-  if (model == kPotts) return launch_pdl(k_apply<kPotts>, g, kFlipThreads, st, lat, sweep, m, count);
-  if (model == kClock) return launch_pdl(k_apply<kClock>, g, kFlipThreads, st, lat, sweep, m, count);
-  return launch_pdl(k_apply<kXY>, g, kFlipThreads, st, lat, sweep, m, count);
+  static_assert(kFlipWalkSites >= 32 * 256, "a one-tile lattice walks");
+  if (finalize && one_tile(lat))  // else the merge has written it
+    return launch_pdl(k_apply<MODEL, true, true>, g + 1u, kFlipThreads, st, lat, sweep, m, count, finalize);
+  finalize = 0u;
+  if (flip_walks(lat)) return launch_pdl(k_apply<MODEL, true, false>, g, kFlipThreads, st, lat, sweep, m, count, finalize);
+  return launch_pdl(k_apply<MODEL, false, false>, g, kFlipThreads, st, lat, sweep, m, count, finalize);
+}
+
+}  // namespace
+
+namespace {
+template <int D>
+cudaError_t launch_merge_dim(const Lattice& lat, const Measure& m, uint32_t finalize, unsigned g, cudaStream_t st) {
+  constexpr unsigned t = (unsigned)Tile<D>::THREADS;
+  switch (tile_split(lat)) {
+    case 4: return launch_pdl(k_merge<D, 4>, g, 4 * t, st, lat, m, finalize);
+    case 2: return launch_pdl(k_merge<D, 2>, g, 2 * t, st, lat, m, finalize);
+    default: return launch_pdl(k_merge<D, 1>, g, t, st, lat, m, finalize);
+  }
+}
+}  // namespace
+
+cudaError_t launch_merge(const Lattice& lat, const Measure& m, uint32_t finalize, cudaStream_t st) {
+  if (one_tile(lat)) return cudaSuccess;
+  const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz) + (finalize ? 1u : 0u);
+  Lattice l = lat;
+  if (flip_walks(lat)) l.hooked = nullptr;  // nothing reads the lists
+  return lat.dim == 2 ? launch_merge_dim<2>(l, m, finalize, g, st) : launch_merge_dim<3>(l, m, finalize, g, st);
+}
+
+cudaError_t launch_merge(const Lattice& lat, cudaStream_t st) { return launch_merge(lat, Measure{}, 0u, st); }
+
+cudaError_t launch_flip(const Lattice& lat, int model, uint32_t sweep, const Measure& m, bool count,
+                        uint32_t finalize, cudaStream_t st) {
+  if (!flip_walks(lat)) {
+    const unsigned ntiles = (unsigned)(lat.ntx * lat.nty * lat.ntz);
+    const cudaError_t e = launch_pdl(k_compress, ntiles, kFlipThreads, st, lat);
+    if (e != cudaSuccess) return e;
+  }
+  if (model == kIsing) return launch_apply<kIsing>(lat, sweep, m, count, finalize, st);
+  if (model == kPotts) return launch_apply<kPotts>(lat, sweep, m, count, finalize, st);
+  if (model == kClock) return launch_apply<kClock>(lat, sweep, m, count, finalize, st);
+  return launch_apply<kXY>(lat, sweep, m, count, finalize, st);
 }
 
 namespace {

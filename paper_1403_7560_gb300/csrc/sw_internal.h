@@ -154,6 +154,9 @@ int merge_list_capacity(int dim, int shape = -1);
 // over all tile shapes; for the others, the single-lattice shape's.
 void tile_buffers(int model, int dim, int L, size_t* ntiles, size_t* hook_words);
 
+// Threads per row word (1, 2 or 4) of a single lattice's tile kernels.
+int tile_split(const Lattice& lat);
+
 // Message returned by sw_last_error() on the calling thread.
 void set_last_error(const std::string& msg);
 
@@ -183,10 +186,12 @@ cudaError_t launch_label(const Lattice& lat, uint32_t sweep, bool from_mask, cud
 // sweep - 1) into the record of sweep - 1.
 cudaError_t launch_label_measured(const Lattice& lat, uint32_t sweep, const Measure& m,
                                   cudaStream_t st);
+// Joins the tiles.  With finalize != 0 it and launch_flip, given the same
+// value, also write the record of sweep `finalize` from the sums a previous
+// kernel left in m: the merge where there is one, else the flip.
+cudaError_t launch_merge(const Lattice& lat, const Measure& m, uint32_t finalize, cudaStream_t st);
 cudaError_t launch_merge(const Lattice& lat, cudaStream_t st);
-// Flip of `sweep`; counts roots into m.nclusters[sweep & 1] when `count`;
-// when finalize != 0 its first block first writes the record of sweep
-// `finalize` from the sums a previous kernel left in m.
+// Flip of `sweep`; counts roots into m.nclusters[sweep & 1] when `count`.
 cudaError_t launch_flip(const Lattice& lat, int model, uint32_t sweep, const Measure& m, bool count,
                         uint32_t finalize, cudaStream_t st);
 // Stand-alone measurement of the current spins as the record of `sweep`

@@ -922,8 +922,6 @@ void tiles_for(int dim, int L, int* ntx, int* nty, int* ntz, int shape) {
   *ntz = (dim == 2) ? 1 : (L + tz - 1) / tz;
 }
 
-namespace {
-
 // Threads per row word of a lattice's labeling: the most (4, 2 or 1) with
 // which the GPU holds all tiles at once.  With few tiles the kernel is a chain
 // of latencies -- a thread's three Bernoulli words, its hooks and unions, its
@@ -933,17 +931,19 @@ namespace {
 // 1024 (256 tiles) 31.1 / 27.7 / 27.4, 1448 (552) 36.7 / 33.9 / 38.9; 3D L =
 // 32 29.8 / 27.1 / 26.9, 100 (196 tiles of twice the size) 41.5 / 40.1 /
 // 43.2, 128 (256) 44.2 / 43.1 / 50.1, 161 (726) 68.9 / 71.7 / 84.3.
-template <int D>
-int label_split(const Lattice& lat) {
+int tile_split(const Lattice& lat) {
   const int tiles = lat.ntx * lat.nty * lat.ntz;
-  const int whole = sm_count() * (kLabelSplitThreads / Tile<D>::THREADS);  // tiles held at K = 1
+  const int threads = kShapeTY[lat.dim - 2][kSingleShape[lat.dim - 2]] * kShapeTZ[lat.dim - 2][kSingleShape[lat.dim - 2]];
+  const int whole = sm_count() * (kLabelSplitThreads / threads);  // tiles held at one thread a row word
   return 4 * tiles <= whole ? 4 : 2 * tiles <= whole ? 2 : 1;
 }
+
+namespace {
 
 template <int D, bool FROM_MASK, int MM>
 cudaError_t launch_label_kernel(const Lattice& lat, uint32_t sweep, const Measure& m, cudaStream_t st) {
   const unsigned g = (unsigned)(lat.ntx * lat.nty * lat.ntz), t = (unsigned)Tile<D>::THREADS;
-  switch (label_split<D>(lat)) {
+  switch (tile_split(lat)) {
     case 4: return launch_pdl(k_label<D, 4, FROM_MASK, MM>, g, 4 * t, st, lat, sweep, m);
     case 2: return launch_pdl(k_label<D, 2, FROM_MASK, MM>, g, 2 * t, st, lat, sweep, m);
     default: return launch_pdl(k_label<D, 1, FROM_MASK, MM>, g, t, st, lat, sweep, m);

@@ -121,3 +121,24 @@ def test_tiled_sweeps_split_and_ragged(sw, model, dim, L, q):
     finally:
         sw.sw_destroy(h)
         o.close()
+
+
+@pytest.mark.parametrize("model,dim,L,q", [
+    # one tile (no merge), tiles merged and walked without a compression, the
+    # last size that walks and the first that does not
+    (oracle.CLOCK, 2, 32, 37), (oracle.CLOCK, 3, 16, 512), (oracle.CLOCK, 2, 33, 6), (ISING, 2, 1024, 2),
+    (ISING, 2, 1025, 2), (POTTS, 3, 101, 3), (POTTS, 3, 102, 3)])
+def test_flip_paths(sw, model, dim, L, q):
+    T = 2.27 if model == ISING else 0.9 if model == oracle.CLOCK and dim == 2 else 2.2 if model == oracle.CLOCK else 1.8
+    h = sw.sw_create(model, dim, L, q, T, 11 + L)
+    o = oracle.Oracle(model, dim, L, q, T, 11 + L)
+    try:
+        sw.sw_sweep(h, 3)
+        o.sweep(3)
+        assert np.array_equal(sw.sw_get_labels(h), o.labels)
+        assert np.array_equal(sw.sw_get_spins(h), o.spins)
+        got, ref = sw.sw_measure(h), o.take_acc()
+        assert all(got[f] == ref[f] for f in ref)
+    finally:
+        sw.sw_destroy(h)
+        o.close()
