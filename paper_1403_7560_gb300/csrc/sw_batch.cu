@@ -55,6 +55,7 @@ struct sw_batch {
 namespace {
 
 constexpr uint32_t kSmallChunk = 256;  // sweeps of the small members per launch
+constexpr uint32_t kMeasureAfter = 16;  // sweeps of a call after which its last records are measured at once
 
 int bfail(int code, const std::string& msg) {
   swgb::set_last_error(msg);
@@ -371,6 +372,11 @@ int batch_sweep(sw_batch* b, int n, float* ms) {
   for (uint32_t s = 0; b->ntiles && s < replays && e == cudaSuccess; ++s) e = cudaGraphLaunch(b->graph, b->stream);
   if (e == cudaSuccess && b->n_small) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
   if (e == cudaSuccess && ms) e = cudaEventRecord(t1, b->stream);
+  // the tiled members' last records: left to the next call's first sweep, or,
+  // after many sweeps, measured for all members in one launch (about 20 us)
+  // instead of one launch and 12 us for each that is read
+  const bool measured = b->ntiles && replays >= kMeasureAfter;
+  if (e == cudaSuccess && measured) e = swgb::launch_measure_batch(view(b), b->dim, b->shape, b->ntiles, b->stream);
   // later work on each member waits for the batch
   if (e == cudaSuccess) e = cudaEventRecord(b->ev, b->stream);
   if (e == cudaSuccess) {
@@ -379,9 +385,9 @@ int batch_sweep(sw_batch* b, int n, float* ms) {
       if ((e = cudaStreamWaitEvent(h->stream, b->ev, 0)) != cudaSuccess) break;
       if (count[m] == 0) continue;
       h->sweep += count[m];
-      // a tiled member's last record is written on demand; a small member
-      // writes every record in its sweep
-      if (!b->is_small[m]) h->pending = h->sweep;
+      // a tiled member's last record, if it is not written yet, is written on
+      // demand; a small member writes every record in its sweep
+      if (!b->is_small[m]) h->pending = measured ? 0 : h->sweep;
     }
   }
   if (e == cudaSuccess && ms) e = cudaEventSynchronize(t1);

@@ -223,6 +223,9 @@ cudaError_t launch_merge_batch(const BatchView& bv, int dim, int shape, int sche
 cudaError_t launch_flip_batch(const BatchView& bv, int dim, int shape, int schedule, uint32_t ntiles,
                               cudaStream_t st);
 
+// Writes the last record of every tiled member that had sweeps in this call.
+cudaError_t launch_measure_batch(const BatchView& bv, int dim, int shape, uint32_t ntiles, cudaStream_t st);
+
 // Grid of a persistent launch of kernel k with `threads` threads per CTA
 // over n tile-map entries: the device's SM count times the CTAs of k one SM
 // holds (the occupancy calculator's figure for that kernel), at most n.

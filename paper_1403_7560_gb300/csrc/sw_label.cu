@@ -626,6 +626,63 @@ __global__ void __launch_bounds__(256) k_measure_rows(const __grid_constant__ La
   if (threadIdx.x == 0) *mb.done = 0u;
 }
 
+// Stand-alone measurement of every tiled member of a batch that had sweeps in
+// the current call, as the record of its last one: a CTA per tile-map entry,
+// k_measure_rows' work on the tile's rows; the last of a member's CTAs to
+// finish writes its record.
+template <class S>
+__global__ void __launch_bounds__(S::THREADS) k_measure_batch(BatchView bv) {
+  constexpr int D = S::D, NT = S::THREADS, NW = NT / 32;
+  __shared__ unsigned int s_hist[256];
+  __shared__ unsigned int s_whist[NW * kSmallQ];
+  __shared__ long long s_red[NW];
+  __shared__ double s_rd[NW];
+  __shared__ bool s_last;
+  const BatchMember& m = bv.members[__ldg(&bv.tile_lattice[blockIdx.x])];
+  if (m.nsweeps == 0u) return;  // its record is written, or was pending before the call
+  const Lattice lat = m.lat;    // a private copy: global stores cannot alias it
+  const Measure mb = m.meas;
+  const uint32_t tile = __ldg(&bv.tile_index[blockIdx.x]);
+  const TileCoord tc = tile_coord<S>(lat, tile);
+  const bool potts = lat.model == kPotts;
+  const int L = lat.L, warp = threadIdx.x >> 5;
+  for (int k = threadIdx.x; k < 256; k += NT) s_hist[k] = 0u;
+  for (int k = threadIdx.x; k < NW * kSmallQ; k += NT) s_whist[k] = 0u;
+  __syncthreads();
+  const int r = threadIdx.x, y = tc.y0 + r % S::TY, z = tc.z0 + r / S::TY;
+  int m_acc = 0, e_acc = 0;
+  if (y < L && (D == 2 || z < L)) {
+    const int nvalid = min(32, L - tc.x0);
+    const uint32_t vmask = (nvalid >= 32) ? kFull : ((1u << nvalid) - 1u);
+    const int y1 = (y + 1 == L) ? 0 : y + 1, z1 = (D == 3) ? ((z + 1 == L) ? 0 : z + 1) : 0;
+    RowBytes rb;
+    load_rows<D>(static_cast<const uint8_t*>(lat.spins), L, tc.x0, nvalid, (uint32_t)y + (uint32_t)L * (uint32_t)z,
+                 (uint32_t)y1 + (uint32_t)L * (uint32_t)z, (uint32_t)y + (uint32_t)L * (uint32_t)z1, rb);
+    const uint32_t e0 = eq_bits(rb.a, rb.ax) & vmask;
+    const uint32_t e1 = eq_bits(rb.a, rb.ay) & vmask;
+    const uint32_t e2 = (D == 3) ? (eq_bits(rb.a, rb.az) & vmask) : 0u;
+    if (potts) measure_row<D, 2>(rb, e0, e1, e2, vmask, nvalid, lat.q, m_acc, e_acc, s_whist + warp * kSmallQ, s_hist);
+    else measure_row<D, 1>(rb, e0, e1, e2, vmask, nvalid, lat.q, m_acc, e_acc, s_whist + warp * kSmallQ, s_hist);
+  }
+  if (potts) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < kSmallQ; k += NT)
+      for (int w = 0; w < NW; ++w) s_hist[k] += s_whist[w * kSmallQ + k];
+    __syncthreads();
+    add_histogram(lat, mb, tile, s_hist);
+  }
+  add_integer_sums<NW>(mb, tile, (long long)m_acc, (long long)e_acc, s_red);
+  // this CTA's slot additions are visible before it counts itself done
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(mb.done, 1u) == (uint32_t)(lat.ntx * lat.nty * lat.ntz) - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  finalize_record<NW>(lat, mb, m.sweep0 + m.nsweeps, s_red, s_rd);
+  if (threadIdx.x == 0) *mb.done = 0u;
+}
+
 // ---------------------------------------------------------------- XY bonds
 // 1 + the top 23 bits of w as a fraction (a bit pattern: no conversion, which
 // would share the exp's pipe).
@@ -1011,6 +1068,22 @@ cudaError_t launch_label_batch(const BatchView& bv, int dim, int shape, int sche
   static_assert(kTileShapes == 3, "one instantiation per shape");
   if (dim == 2) return label_batch_dim<2>(bv, shape, schedule, ising_tiles, potts_tiles, st);
   return label_batch_dim<3>(bv, shape, schedule, ising_tiles, potts_tiles, st);
+}
+
+cudaError_t launch_measure_batch(const BatchView& bv, int dim, int shape, uint32_t ntiles, cudaStream_t st) {
+  static_assert(kTileShapes == 3, "one instantiation per shape");
+  auto one = [&](auto kernel, int threads) {
+    kernel<<<ntiles, (unsigned)threads, 0, st>>>(bv);
+    return cudaGetLastError();
+  };
+  if (dim == 2) {
+    if (shape == 1) return one(k_measure_batch<ShapeOf<2, 1>>, ShapeOf<2, 1>::THREADS);
+    if (shape == 2) return one(k_measure_batch<ShapeOf<2, 2>>, ShapeOf<2, 2>::THREADS);
+    return one(k_measure_batch<ShapeOf<2, 0>>, ShapeOf<2, 0>::THREADS);
+  }
+  if (shape == 1) return one(k_measure_batch<ShapeOf<3, 1>>, ShapeOf<3, 1>::THREADS);
+  if (shape == 2) return one(k_measure_batch<ShapeOf<3, 2>>, ShapeOf<3, 2>::THREADS);
+  return one(k_measure_batch<ShapeOf<3, 0>>, ShapeOf<3, 0>::THREADS);
 }
 
 cudaError_t launch_measure_rows(const Lattice& lat, uint32_t sweep, const Measure& m, cudaStream_t st) {

@@ -142,3 +142,38 @@ def test_flip_paths(sw, model, dim, L, q):
     finally:
         sw.sw_destroy(h)
         o.close()
+
+
+@pytest.mark.parametrize("dim,shape", [(2, 0), (2, 1), (2, 2), (3, 0), (3, 1), (3, 2)])
+def test_batch_records_measured_together(sw, dim, shape):
+    """A call of many sweeps measures its members' last records in one launch
+    (rows at every alignment, q on both sides of the per-warp histogram), and
+    a short call leaves them to the next one."""
+    spec = [(ISING, dim, 120 if dim == 2 else 24, 2, 2.3 if dim == 2 else 4.5, 1),
+            (POTTS, dim, 131 if dim == 2 else 27, 3, 1.0, 2), (POTTS, dim, 146 if dim == 2 else 30, 17, 0.7, 3),
+            (ISING, dim, 161 if dim == 2 else 33, 2, 2.2 if dim == 2 else 4.4, 4)]
+    b = sw.sw_batch_create(dim)
+    hs = [sw.sw_create(*s) for s in spec]
+    try:
+        for h in hs:
+            sw.sw_batch_add(b, h)
+        sw.sw_batch_set_config(b, shape, 0)
+        sw.sw_set_sweep_target(hs[3], 12)
+        for n in (17, 3, 16):
+            sw.sw_batch_sweep(b, n)
+        for h, s in zip(hs, spec):
+            n = 12 if h is hs[3] else 36
+            o = oracle.Oracle(*s)
+            o.sweep(n)
+            assert sw.sw_sweep_counter(h) == n
+            assert np.array_equal(sw.sw_get_spins(h), o.spins)
+            ref, last = o.take_acc(), o.last_record()
+            r = sw.sw_get_series(h, n, 1)[0]
+            assert all(r[f] == last[f] for f in last if f in r), (r, last)
+            got = sw.sw_measure(h)
+            assert all(got[f] == ref[f] for f in ref), s
+            o.close()
+    finally:
+        sw.sw_batch_destroy(b)
+        for h in hs:
+            sw.sw_destroy(h)
