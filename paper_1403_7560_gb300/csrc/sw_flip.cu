@@ -258,10 +258,11 @@ __global__ void __launch_bounds__(kCompressThreads, PERSISTENT ? 16 : 24) k_comp
 
 // The words of four consecutive sites' cluster roots, from their own words:
 // the walks take each step together (the forest is read-only here; L1 serves
-// the nodes that a warp's walks share).  Returns how many are roots.
-__device__ __forceinline__ int walk_roots(const Lattice& lat, uint32_t i0, uint32_t* v) {
+// the nodes that a warp's walks share).  at: the roots.  Returns how many of
+// the sites are roots.
+__device__ __forceinline__ int walk_roots(const Lattice& lat, uint32_t i0, uint32_t* v, uint32_t* at) {
   const int shift = lat.sbits + 1;
-  uint32_t at[4], moved = 0u;
+  uint32_t moved = 0u;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     at[j] = i0 + (uint32_t)j;
@@ -360,7 +361,10 @@ __global__ void __launch_bounds__(kFlipThreads) k_apply(Lattice lat, uint32_t sw
       if (!(v[j] & lr_bit)) v[j] = __ldg(&lat.forest[v[j] >> shift]);
       else if ((v[j] >> shift) == 4u * q + (uint32_t)j) ++roots;  // a cluster's root
     }
-    if (WALK) roots += walk_roots(lat, 4u * q, v);
+    if (WALK) {
+      uint32_t at[4];
+      roots += walk_roots(lat, 4u * q, v, at);
+    }
     uint32_t n[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) n[j] = update(old[j], v[j] & dmask);
@@ -506,9 +510,26 @@ __global__ void k_advance(uint32_t* step) {
   *step += 1u;
 }
 
-__global__ void __launch_bounds__(256) k_labels_out(Lattice lat, int32_t* out) {
-  const int shift = lat.sbits + 1;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < lat.N; i += gridDim.x * blockDim.x) {
+// Canonical labels: four sites a thread walk to their roots together, a
+// 16-byte store where the caller's buffer allows it (2^21 sites near the
+// percolation threshold: 15.8 us with a site a thread, 12.2 so).
+__global__ void __launch_bounds__(256) k_labels_out(Lattice lat, int32_t* out, bool vec) {
+  const uint32_t nq = lat.N >> 2;
+  const uint4* f4 = reinterpret_cast<const uint4*>(lat.forest);
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
+    const uint4 w4 = __ldg(&f4[q]);
+    uint32_t v[4] = {w4.x, w4.y, w4.z, w4.w}, at[4];
+    walk_roots(lat, 4u * q, v, at);
+    if (vec) {
+      reinterpret_cast<uint4*>(out)[q] = make_uint4(at[0], at[1], at[2], at[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) out[4u * q + (uint32_t)j] = (int32_t)at[j];
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x < (lat.N & 3u)) {
+    const int shift = lat.sbits + 1;
+    const uint32_t i = 4u * nq + threadIdx.x;
     uint32_t r = lat.forest[i] >> shift;
     uint32_t it = 0;
     for (; it < lat.cap; ++it) {
@@ -681,9 +702,11 @@ cudaError_t launch_advance(const BatchView& bv, cudaStream_t st) {
 }
 
 cudaError_t launch_labels_out(const Lattice& lat, int32_t* out, cudaStream_t st) {
-  unsigned g = (lat.N + 255u) / 256u;
+  unsigned g = (lat.N / 4u + 255u) / 256u;
   if (g > 4096u) g = 4096u;
-  k_labels_out<<<g, 256, 0, st>>>(lat, out);
+  if (g == 0) g = 1;
+  const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  k_labels_out<<<g, 256, 0, st>>>(lat, out, vec);
   return cudaGetLastError();
 }
 

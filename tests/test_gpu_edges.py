@@ -177,3 +177,19 @@ def test_batch_records_measured_together(sw, dim, shape):
         sw.sw_batch_destroy(b)
         for h in hs:
             sw.sw_destroy(h)
+
+
+@pytest.mark.parametrize("dim,L", [(2, 7), (2, 64), (3, 9), (3, 32)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_labels_into_any_buffer(sw, dim, L, offset):
+    """Canonical labels by four sites a thread, into a buffer that is or is
+    not 16-byte aligned; N a multiple of 4 or not."""
+    import torch
+    m = inputs.random_mask(dim, L, 0.4, seed=L)
+    dm = torch.from_numpy(m.view(np.int32).copy()).cuda()
+    out = torch.full((L ** dim + 8,), -1, dtype=torch.int32, device="cuda")
+    sw.sw_label_from_bonds_noalloc(dim, L, dm.data_ptr(), out.data_ptr() + 4 * offset,
+                                   torch.cuda.current_stream().cuda_stream)
+    got = out.cpu().numpy()
+    assert np.array_equal(got[offset:offset + L ** dim], oracle.labels(dim, L, m))
+    assert (got[offset + L ** dim:] == -1).all() and (got[:offset] == -1).all()
