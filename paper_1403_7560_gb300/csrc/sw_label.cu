@@ -731,22 +731,28 @@ struct XYBlock<3> {
 // depends on the grid.
 constexpr int kXYBlocksPerSM[2] = {6, 5};
 
-template <int D, bool MEASURE>
-__global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
+// K > 1: K times the threads for lattices with fewer blocks than SMs, where
+// the kernel is one warp's chain of rows.  A block's rows are dealt to the K
+// sets of warps; the first set then adds the moments alone, in K = 1's order,
+// so the sums are the same bits.  3D L = 16 (two blocks): 18.0 -> 10.5 us, 22.4
+// -> 16.5 with the moments.
+template <int D, int K, bool MEASURE>
+__global__ void __launch_bounds__(256 * K, K == 1 ? kXYBlocksPerSM[D - 2] : 1)
     k_bonds_xy(const __grid_constant__ Lattice lat, uint32_t sweep, const __grid_constant__ Measure mb) {
   constexpr int BY = XYBlock<D>::BY, BZ = XYBlock<D>::BZ;
   constexpr int HX = 33, HY = BY + 1, HZ = (D == 3) ? BZ + 1 : 1, NBOX = HX * HY * HZ;
   constexpr int NW = 256 / 32, RW = BY * BZ / NW;  // rows per warp
-  static_assert(BY % NW == 0 && RW <= 32 && HY >= NW, "a lane per row of the warp");
+  static_assert(BY % NW == 0 && RW <= 32 && RW % K == 0, "a lane per row of the warp");
   __shared__ float2 sv[NBOX];
   __shared__ float s_phi;
-  __shared__ double s_rd[NW];
+  __shared__ double s_rd[K * NW];
   if (threadIdx.x == 0) s_phi = xy_phi(lat, sweep);
   pdl_wait();
   __syncthreads();
   const float phi = s_phi;
   const float kexp = -__fmul_rn(lat.twoK, 0x1.715476p+0f);  // -2K log2 e
-  const int L = lat.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int L = lat.L, lane = threadIdx.x & 31, warp = K == 1 ? threadIdx.x >> 5 : (threadIdx.x >> 5) & (NW - 1);
+  const int set = K == 1 ? 0 : threadIdx.x / (32 * NW);
   const uint32_t plane = lat.R * (uint32_t)lat.W;
   const float* th = static_cast<const float*>(lat.spins);
   const uint32_t nbx = (uint32_t)lat.W, nby = (uint32_t)((L + BY - 1) / BY);
@@ -770,16 +776,24 @@ __global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
     // a warp per halo row (yy, zz), lanes along x; then the +x halo column
     // (entry 32 of every row) a thread per row
     if (lane <= nx)
-      for (int yy = warp, zz = 0; zz < HZ && zz <= nz;) {
+      for (int yy = K == 1 ? warp : (warp + NW * set) % HY, zz = K == 1 ? 0 : (warp + NW * set) / HY;
+           zz < HZ && zz <= nz;) {
         if (yy <= ny) project(yy, zz, lane);
-        yy += NW;
-        if (yy >= HY) {
-          yy -= HY;
-          ++zz;
+        yy += K * NW;
+        if (K == 1) {
+          if (yy >= HY) {
+            yy -= HY;
+            ++zz;
+          }
+        } else {
+          while (yy >= HY) {
+            yy -= HY;
+            ++zz;
+          }
         }
       }
     if (nx == 32)
-      for (int hr = threadIdx.x; hr < HY * HZ; hr += 256) {
+      for (int hr = threadIdx.x; hr < HY * HZ; hr += 256 * K) {
         const int yy = hr % HY, zz = hr / HY;
         if (yy <= ny && zz <= nz) project(yy, zz, 32);
       }
@@ -792,7 +806,7 @@ __global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
     const uint32_t i0 = (uint32_t)(x0 + lane) + (uint32_t)L * ((uint32_t)(y0 + warp) + (uint32_t)L * (uint32_t)z0);
     constexpr int RY = BY / NW;  // rows of the warp per z
 #pragma unroll 2
-    for (int k = 0; k < RW; ++k) {
+    for (int k = set; k < RW; k += K) {
       const int yy = warp + NW * (k % RY), zz = k / RY;
       bool act[D];
 #pragma unroll
@@ -817,9 +831,9 @@ __global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
             const float u = __fmul_rn((float)(word_of(w, d) >> 8), 0x1p-24f);
             act[d] = u < -expm1f(-__fmul_rn(lat.twoK, prod));
           }
-          if (MEASURE) fe = __fadd_rn(fe, __fadd_rn(prod, __fmul_rn(si.y, sj.y)));
+          if (MEASURE && K == 1) fe = __fadd_rn(fe, __fadd_rn(prod, __fmul_rn(si.y, sj.y)));
         }
-        if (MEASURE) {
+        if (MEASURE && K == 1) {
           fx = __fadd_rn(fx, si.x);
           fy = __fadd_rn(fy, si.y);
         }
@@ -832,10 +846,26 @@ __global__ void __launch_bounds__(256, kXYBlocksPerSM[D - 2])
     }
     {
       const int yy = warp + NW * (lane % RY), zz = lane / RY;
-      if (lane < RW && yy < ny && zz < nz) {
+      if (lane < RW && (K == 1 || lane % K == set) && yy < ny && zz < nz) {
         const uint32_t g = ((uint32_t)(y0 + yy) + (uint32_t)L * (uint32_t)(z0 + zz)) * (uint32_t)lat.W + (uint32_t)(x0 >> 5);
 #pragma unroll
         for (int d = 0; d < D; ++d) lat.planes[d * plane + g] = m[d];
+      }
+    }
+    if (MEASURE && K > 1 && set == 0 && lane < nx) {
+#pragma unroll 2
+      for (int k = 0; k < RW; ++k) {
+        const int yy = warp + NW * (k % RY), zz = k / RY;
+        if (yy >= ny || zz >= nz) continue;
+        const int c = lane + HX * (yy + HY * zz);
+        const float2 si = sv[c];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const float2 sj = sv[c + (d == 0 ? 1 : d == 1 ? HX : HX * HY)];
+          fe = __fadd_rn(fe, __fadd_rn(__fmul_rn(si.x, sj.x), __fmul_rn(si.y, sj.y)));
+        }
+        fx = __fadd_rn(fx, si.x);
+        fy = __fadd_rn(fy, si.y);
       }
     }
   }
@@ -957,18 +987,15 @@ __global__ void __launch_bounds__(256) k_bonds_clock(const __grid_constant__ Lat
 
 cudaError_t launch_bonds_clock(const Lattice& lat, uint32_t sweep, const Measure* m, cudaStream_t st) {
   const uint32_t words = lat.R * (uint32_t)lat.W;
-  unsigned g = (words + 7u) / 8u;
-  if (g > 4096u) g = 4096u;
-  cudaError_t e = cudaSuccess;
+  // one wave of CTAs (each fills its tables, 12 KB at q = 512, once), a warp
+  // per row word striding over them; the sums are exact integers, so the grid
+  // changes no result.  3D q = 512 L = 128, 4096 CTAs / one wave: 34.3 / 31.5 us
+  auto launch = [&](auto kernel, const Measure& mm) {
+    return launch_pdl(kernel, batch_grid(kernel, 256, (words + 7u) / 8u), 256, st, lat, sweep, mm);
+  };
   const Measure none{};
-  if (lat.dim == 2) {
-    if (m) e = launch_pdl(k_bonds_clock<2, true>, g, 256, st, lat, sweep, *m);
-    else e = launch_pdl(k_bonds_clock<2, false>, g, 256, st, lat, sweep, none);
-  } else {
-    if (m) e = launch_pdl(k_bonds_clock<3, true>, g, 256, st, lat, sweep, *m);
-    else e = launch_pdl(k_bonds_clock<3, false>, g, 256, st, lat, sweep, none);
-  }
-  return e;
+  if (lat.dim == 2) return m ? launch(k_bonds_clock<2, true>, *m) : launch(k_bonds_clock<2, false>, none);
+  return m ? launch(k_bonds_clock<3, true>, *m) : launch(k_bonds_clock<3, false>, none);
 }
 
 void tiles_for(int dim, int L, int* ntx, int* nty, int* ntz, int shape) {
@@ -1121,20 +1148,22 @@ cudaError_t launch_bonds_xy(const Lattice& lat, uint32_t sweep, const Measure* m
   // one wave: the CTAs the GPU holds at once, each striding over the blocks;
   // at most kMeasureBlocks (the slots of the XY partials)
   unsigned g = 0;
-  auto launch = [&](auto kernel, const Measure& mm) {
-    g = (unsigned)(sm_count() * kXYBlocksPerSM[lat.dim - 2]);
-    if (g > nb) g = nb;
-    if (g > (unsigned)kMeasureBlocks) g = (unsigned)kMeasureBlocks;
-    return launch_pdl(kernel, g, 256, st, lat, sweep, mm);
+  g = (unsigned)(sm_count() * kXYBlocksPerSM[lat.dim - 2]);
+  if (g > nb) g = nb;
+  if (g > (unsigned)kMeasureBlocks) g = (unsigned)kMeasureBlocks;
+  // the threads of four blocks for each where every block has an SM of its own
+  const bool split = nb <= (uint32_t)sm_count();
+  auto launch = [&](auto kernel, auto wide, const Measure& mm) {
+    return split ? launch_pdl(wide, g, 1024, st, lat, sweep, mm) : launch_pdl(kernel, g, 256, st, lat, sweep, mm);
   };
   cudaError_t e = cudaSuccess;
   const Measure none{};
   if (lat.dim == 2) {
-    if (m) e = launch(k_bonds_xy<2, true>, *m);
-    else e = launch(k_bonds_xy<2, false>, none);
+    if (m) e = launch(k_bonds_xy<2, 1, true>, k_bonds_xy<2, 4, true>, *m);
+    else e = launch(k_bonds_xy<2, 1, false>, k_bonds_xy<2, 4, false>, none);
   } else {
-    if (m) e = launch(k_bonds_xy<3, true>, *m);
-    else e = launch(k_bonds_xy<3, false>, none);
+    if (m) e = launch(k_bonds_xy<3, 1, true>, k_bonds_xy<3, 4, true>, *m);
+    else e = launch(k_bonds_xy<3, 1, false>, k_bonds_xy<3, 4, false>, none);
   }
   if (blocks) *blocks = (int)g;
   return e;
