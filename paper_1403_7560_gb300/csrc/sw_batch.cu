@@ -8,7 +8,9 @@
 // and in any batch.  Measurement follows the single-lattice scheme: the
 // labeling kernel of sweep k measures the state after sweep k-1 and the
 // compression kernel's first tile of each member writes that record; the
-// last sweep of a call stays pending on the handle.
+// last sweep of a short call stays pending on the handle, that of a long one
+// is measured for all members in one launch.  Small members run all sweeps
+// of a call in a launch of their own beside the graph's replays.
 #include <algorithm>
 #include <new>
 #include <string>

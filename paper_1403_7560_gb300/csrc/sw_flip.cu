@@ -10,8 +10,9 @@
 // k_merge: bonds that leave a tile join the local roots at their two ends
 //   with atomicMin hooking of the larger root under the smaller; a warp
 //   performs each distinct (root, root) pair once.
-// k_merge also lists, per tile, the roots it hooked under another tree.
-// k_compress: every listed root walks to its global root (the smallest site
+// k_merge also lists, per tile, the roots it hooked under another tree, and
+//   its first CTA writes the previous sweep's record.
+// k_compress (above kFlipWalkSites sites): every listed root walks to its global root (the smallest site
 //   index of the cluster), takes that root's draw and stores (root, draw) in
 //   its own word.
 // k_apply: every site reads its local root's word (or its own) and writes
