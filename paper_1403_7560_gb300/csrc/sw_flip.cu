@@ -229,16 +229,26 @@ __global__ void __launch_bounds__(kFlipThreads, 8) k_compress(Lattice lat) {
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) compress_tile(lat, t);
 }
 
+// Threads of a batch compression CTA, by the most roots that a tile of the
+// shape can list: a 2D tile lists some tens, and small CTAs keep more tiles'
+// walks in flight (4459 tiles: 23.7 us with 256 threads, 17.0 with 64); a 3D
+// tile lists hundreds, and 64 threads take them in many rounds.  us per batch
+// sweep with 64 / 128 / 256 threads: eight 2D Ising L = 1024 80.1 / 80.1 /
+// 82.3, 300 of L = 200 138.9 / 140.4 / 144.2; 3D tiles of 16 x 16, eight L =
+// 64 60.0 / 55.0 / 53.6, 150 of L = 40 166.1 / 164.6 / 164.8; of 16 x 8 56.8 /
+// 53.6 / 52.4, 159.6 / 158.6 / 161.2; of 8 x 8 59.8 / 58.4 / 58.2, 161.5 /
+// 161.9 / 167.9.
+template <class S>
+constexpr int compress_threads() {
+  return MergeShape<S>::kMax >= 800 ? 256 : MergeShape<S>::kMax >= 400 ? 128 : 64;
+}
+
 // Batch: one CTA per member tile; the CTA of each member's tile 0 first
 // writes that member's previous record (every step after the first).
-// Threads of a batch compression CTA: a tile lists some tens of hooked roots
-// (2D), and smaller CTAs keep more tiles' walks in flight (4459 tiles: 23.7 us
-// with 256 threads, 17.0 with 64).
-constexpr int kCompressThreads = 64, kCompressWarps = kCompressThreads / 32;
-template <bool PERSISTENT>
-__global__ void __launch_bounds__(kCompressThreads, PERSISTENT ? 16 : 24) k_compress_batch(BatchView bv, uint32_t n) {
-  __shared__ long long s_red[kCompressWarps];
-  __shared__ double s_rd[kCompressWarps];
+template <int NT, bool PERSISTENT>
+__global__ void __launch_bounds__(NT, (PERSISTENT ? 1024 : 1536) / NT) k_compress_batch(BatchView bv, uint32_t n) {
+  __shared__ long long s_red[NT / 32];
+  __shared__ double s_rd[NT / 32];
   pdl_wait();
   const uint32_t step = *bv.step;
   auto entry = [&](uint32_t t) {
@@ -247,7 +257,7 @@ __global__ void __launch_bounds__(kCompressThreads, PERSISTENT ? 16 : 24) k_comp
     if (step >= m.nsweeps) return;
     const Lattice lat = m.lat;  // a private copy: global stores cannot alias it
     if (tile == 0u && (step > 0u || m.measure0))
-      finalize_record<kCompressWarps>(lat, m.meas, m.sweep0 + step, s_red, s_rd);
+      finalize_record<NT / 32>(lat, m.meas, m.sweep0 + step, s_red, s_rd);
     compress_tile(lat, tile);
   };
   if constexpr (PERSISTENT) {
@@ -652,15 +662,16 @@ cudaError_t merge_batch_shape(const BatchView& bv, uint32_t ntiles, bool persist
 template <int D, int SH>
 cudaError_t flip_batch_shape(const BatchView& bv, uint32_t ntiles, bool persistent, cudaStream_t st) {
   using S = ShapeOf<D, SH>;
+  constexpr int kCompress = compress_threads<S>();
   cudaError_t e;
   if (!persistent) {
-    e = launch_pdl(k_compress_batch<false>, ntiles, kCompressThreads, st, bv, ntiles);
+    e = launch_pdl(k_compress_batch<kCompress, false>, ntiles, kCompress, st, bv, ntiles);
     if (e == cudaSuccess) e = launch_pdl(k_apply_batch<S, false>, ntiles, kFlipThreads, st, bv, ntiles);
     return e;
   }
-  const unsigned gc = batch_grid(k_compress_batch<true>, kCompressThreads, ntiles);
+  const unsigned gc = batch_grid(k_compress_batch<kCompress, true>, kCompress, ntiles);
   const unsigned ga = batch_grid(k_apply_batch<S, true>, kFlipThreads, ntiles);
-  e = launch_pdl(k_compress_batch<true>, gc, kCompressThreads, st, bv, ntiles);
+  e = launch_pdl(k_compress_batch<kCompress, true>, gc, kCompress, st, bv, ntiles);
   if (e == cudaSuccess) e = launch_pdl(k_apply_batch<S, true>, ga, kFlipThreads, st, bv, ntiles);
   return e;
 }
