@@ -987,11 +987,19 @@ __global__ void __launch_bounds__(256) k_bonds_clock(const __grid_constant__ Lat
 
 cudaError_t launch_bonds_clock(const Lattice& lat, uint32_t sweep, const Measure* m, cudaStream_t st) {
   const uint32_t words = lat.R * (uint32_t)lat.W;
-  // one wave of CTAs (each fills its tables, 12 KB at q = 512, once), a warp
-  // per row word striding over them; the sums are exact integers, so the grid
-  // changes no result.  3D q = 512 L = 128, 4096 CTAs / one wave: 34.3 / 31.5 us
+  // a warp per row word, striding over them; the sums are exact integers, so
+  // the grid changes no result.  Few row words: one wave of CTAs, each filling
+  // its tables (12 KB at q = 512) once; many: up to 4096 CTAs, whose unequal
+  // ends the next ones fill.  us per measured sweep, one wave / 4096: 3D L = 64
+  // q = 512 (8192 row words) 28.1 / 29.3, 128 (65536) 58.5 / 60.5, 2D L = 1448
+  // (66608) 53.3 / 56.5, 3D q = 6 L = 129 (83205) 74.9 / 75.5, 144 (103680) 82.5
+  // / 81.6, 160 (128000) 97.7 / 95.1, 200 (280000) 179.1 / 170.6, 400 1177 /
+  // 1100; 2D L = 8000 974 / 892.
+  constexpr uint32_t kWaveWords = 3u << 15;
+  const uint32_t ctas = (words + 7u) / 8u;
   auto launch = [&](auto kernel, const Measure& mm) {
-    return launch_pdl(kernel, batch_grid(kernel, 256, (words + 7u) / 8u), 256, st, lat, sweep, mm);
+    const unsigned g = words <= kWaveWords ? batch_grid(kernel, 256, ctas) : ctas < 4096u ? ctas : 4096u;
+    return launch_pdl(kernel, g, 256, st, lat, sweep, mm);
   };
   const Measure none{};
   if (lat.dim == 2) return m ? launch(k_bonds_clock<2, true>, *m) : launch(k_bonds_clock<2, false>, none);
