@@ -893,8 +893,14 @@ __global__ void __launch_bounds__(256 * K, K == 1 ? kXYBlocksPerSM[D - 2] : 1)
 // With MEASURE the same loads measure the incoming state: integer sums of
 // the fixed-point tables C[p_i], S[p_i] and C[(p_i - p_j) mod q], added to
 // the clock slots per block.
+//
+// CTAs per SM of the one-wave grid, update only and measured: what registers
+// (32 and 40) and shared memory (8 and 24 KB) allow.  Fixed, not asked of the
+// occupancy calculator, which every sweep's launch would wait for.
+constexpr int kClockBlocksPerSM[2] = {8, 6};
+
 template <int D, bool MEASURE>
-__global__ void __launch_bounds__(256) k_bonds_clock(const __grid_constant__ Lattice lat, uint32_t sweep,
+__global__ void __launch_bounds__(256, kClockBlocksPerSM[MEASURE]) k_bonds_clock(const __grid_constant__ Lattice lat, uint32_t sweep,
                                                       const __grid_constant__ Measure mb) {
   __shared__ uint32_t s_mirror;
   __shared__ long long s_red[256 / 32];
@@ -997,10 +1003,9 @@ cudaError_t launch_bonds_clock(const Lattice& lat, uint32_t sweep, const Measure
   // 1100; 2D L = 8000 974 / 892.
   constexpr uint32_t kWaveWords = 3u << 15;
   const uint32_t ctas = (words + 7u) / 8u;
-  auto launch = [&](auto kernel, const Measure& mm) {
-    const unsigned g = words <= kWaveWords ? batch_grid(kernel, 256, ctas) : ctas < 4096u ? ctas : 4096u;
-    return launch_pdl(kernel, g, 256, st, lat, sweep, mm);
-  };
+  const uint32_t most = words <= kWaveWords ? (uint32_t)(sm_count() * kClockBlocksPerSM[m != nullptr]) : 4096u;
+  const unsigned g = ctas < most ? ctas : most;
+  auto launch = [&](auto kernel, const Measure& mm) { return launch_pdl(kernel, g, 256, st, lat, sweep, mm); };
   const Measure none{};
   if (lat.dim == 2) return m ? launch(k_bonds_clock<2, true>, *m) : launch(k_bonds_clock<2, false>, none);
   return m ? launch(k_bonds_clock<3, true>, *m) : launch(k_bonds_clock<3, false>, none);
