@@ -369,10 +369,16 @@ int batch_sweep(sw_batch* b, int n, float* ms) {
     for (uint32_t s = 0; s < replays && e == cudaSuccess; s += kSmallChunk)
       e = swgb::launch_small_batch(b->d_members, b->dim, b->d_small, b->n_small, b->small_smem, s, kSmallChunk,
                                    b->side);
-    if (e == cudaSuccess) e = cudaEventRecord(b->ev_join, b->side);
   }
   for (uint32_t s = 0; b->ntiles && s < replays && e == cudaSuccess; ++s) e = cudaGraphLaunch(b->graph, b->stream);
-  if (e == cudaSuccess && b->n_small) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+  if (b->n_small) {
+    // after a failed launch too: whoever waits for the batch stream (a member
+    // leaving, sw_batch_destroy before it frees the descriptors) then waits
+    // for the side stream's sweeps
+    cudaError_t j = cudaEventRecord(b->ev_join, b->side);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+    if (e == cudaSuccess) e = j;
+  }
   if (e == cudaSuccess && ms) e = cudaEventRecord(t1, b->stream);
   // the tiled members' last records: left to the next call's first sweep, or,
   // after many sweeps, measured for all members in one launch (about 20 us)
