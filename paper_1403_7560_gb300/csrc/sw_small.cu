@@ -586,14 +586,27 @@ cudaError_t launch_small_t(const Lattice& lat, const Measure& m, uint32_t sweep0
   return cudaGetLastError();
 }
 
+// Two CTAs of `smem` bytes of dynamic shared memory on one SM (228 KB, of which
+// each CTA takes its static part and 1 KB besides, in units of 128 bytes).
+bool two_fit(size_t smem) {
+  const size_t cta = ((smem + sizeof(SmallScratch) + sizeof(Lattice) + 127) & ~(size_t)127) + 1024;
+  return 2 * cta <= 228 * 1024;
+}
+
 template <int D>
 cudaError_t launch_small_batch_t(const BatchMember* members, const uint32_t* list, uint32_t count, size_t smem,
                                  uint32_t first, uint32_t n, cudaStream_t st) {
   static thread_local int configured_device = -1;
   const cudaError_t e = allow_small_smem(k_sweep_small_batch<D>, configured_device);
   if (e != cudaSuccess) return e;
-  // members beyond one CTA per SM share SMs in pairs of half-size CTAs
-  const unsigned threads = count <= (uint32_t)sm_count() ? kSmallThreads : kSmallThreads / 2;
+  // members beyond one CTA per SM share SMs in pairs of half-size CTAs, where
+  // an SM's shared memory holds two of the largest; else each has an SM to
+  // itself and all of its threads.  us per batch sweep of 300 members, 512 /
+  // 1024 threads: pairs fit, 2D Ising L = 64 18.9 / 23.5, 104 36.4 / 43.1, 3D
+  // 18 39.0 / 43.5; they do not, 2D 112 49.6 / 44.2, Potts q = 3 L = 100 60.6
+  // / 53.8, 3D 20 56.6 / 50.6, 300 of L = 64 and one of 112 37.0 / 34.0
+  const bool pairs = count > (uint32_t)sm_count() && two_fit(smem);
+  const unsigned threads = pairs ? kSmallThreads / 2 : kSmallThreads;
   k_sweep_small_batch<D><<<count, threads, smem, st>>>(members, list, first, n);
   return cudaGetLastError();
 }
