@@ -570,12 +570,21 @@ def _job_list(specs):
     return [Job(**d) for d in specs]
 
 
+# The library's batch rules (sw_internal.h, sw_batch.cu): sites up to which a
+# member runs whole in one CTA, sweeps of such members per launch, and sweeps
+# of a call from which its last records are measured at its end.
+SMALL_SITES = {2: 12544, 3: 10648}
+SMALL_CHUNK = 256
+MEASURE_AFTER = 16
+
+
 def batch_launches(specs, schedule):
     """Kernels of one batch sweep, a launch per phase: the tiled members' labels (one
     launch per model under label layout 0, one in all under layout 1 -- bit 0
     of the schedule), merge (one launch, or one per axis under bit 2),
-    compression and apply; one launch per model of the small members (2D up
-    to 8192 sites, 3D up to 4096); the step counter."""
+    compression and apply; the step counter.  Members of up to 8192 sites (2D)
+    or 4096 (3D) count as one launch per model: the library runs them apart
+    from the sweeps, which batch_call_launches counts."""
     def is_small(m, d, L):
         return L ** d <= (8192 if d == 2 else 4096)
     tiled = {m for (m, d, L, _, _, _) in specs if not is_small(m, d, L)}
@@ -589,11 +598,12 @@ def batch_launches(specs, schedule):
 def batch_call_launches(specs, schedule, sweeps):
     """Kernels one sw_batch_sweep(b, sweeps) launches: per sweep the tiled
     members' labels, merge, compression, apply and the step counter
-    (batch_launches without small members); for the small members (2D up to
-    12544 sites, 3D up to 10648) one launch per 256 sweeps."""
-    tiled = [x for x in specs if x[2] ** x[1] > (12544 if x[1] == 2 else 10648)]
-    n = batch_launches(tiled, schedule) * sweeps if tiled else 0
-    return n + (-(-sweeps // 256) if len(tiled) < len(specs) else 0)
+    (batch_launches without small members), and from MEASURE_AFTER sweeps on
+    one measurement of their last states; for the small members one launch per
+    SMALL_CHUNK sweeps."""
+    tiled = [x for x in specs if x[2] ** x[1] > SMALL_SITES[x[1]]]
+    n = batch_launches(tiled, schedule) * sweeps + (sweeps >= MEASURE_AFTER) if tiled else 0
+    return n + (-(-sweeps // SMALL_CHUNK) if len(tiled) < len(specs) else 0)
 
 
 def small_batch(sw, inputs, st, sweeps=50):
