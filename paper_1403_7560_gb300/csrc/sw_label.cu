@@ -828,8 +828,9 @@ __global__ void __launch_bounds__(256 * K, K == 1 ? kXYBlocksPerSM[D - 2] : 1)
           const float prod = __fmul_rn(si.x, sj.x);
           // u < p with p = -expm1f(-2K prod), u = (w >> 8) 2^-24: the sign
           // of (1 + u) + exp(-2K prod) - 2 decides, with u cut to 23 bits
-          // and a fast exp, unless it lies within a margin far above their
-          // error (2^-23 and a few ulp), where expm1f decides
+          // and the hardware's 2^x, unless it lies within a margin far above
+          // their error (below 5.5e-7, as for the clock bonds), where expm1f
+          // decides
           const float near = __fsub_rn(
               __fadd_rn(unit_bits(word_of(w, d)), fast_exp2(__fmul_rn(kexp, prod))), 2.0f);
           act[d] = prod > 0.0f && near < 0.0f;
@@ -892,10 +893,10 @@ __global__ void __launch_bounds__(256 * K, K == 1 ? kXYBlocksPerSM[D - 2] : 1)
 // q-state clock: x_i = sin(pi k_i / q), k_i = (2 p_i - s) mod 2q for the
 // sweep's mirror index s; bond (i,d) active iff u(i,d) < t[k_i][k_j] (the
 // table is 0 where x_i x_j <= 0); u(i,d) = word d of Philox(i, sweep, BOND, 0).
-// The comparison is decided from a float estimate of t (the projections in
-// shared memory, __expf) unless the draw lies within a margin far above the
-// estimate's error, where the exact table entry decides: the result is the
-// table's, without a table gather per bond.
+// The comparison is decided from a float estimate of u - t (the projections in
+// shared memory, the hardware's 2^x) unless it lies within a margin far above
+// the estimate's error, where the exact table entry decides: the result is
+// the table's, without a table gather per bond.
 // With MEASURE the same loads measure the incoming state: integer sums of
 // the fixed-point tables C[p_i], S[p_i] and C[(p_i - p_j) mod q], added to
 // the clock slots per block.
@@ -922,10 +923,12 @@ __global__ void __launch_bounds__(256, kClockBlocksPerSM[MEASURE]) k_bonds_clock
     if (MEASURE) s_fix[k] = __ldg(&mb.cfix[k]);
   }
   __syncthreads();
-  // Error of the float threshold estimate below against the exact table
-  // entry t/2^32 (x rounded to float, products and 2K in float, __expf,
-  // the draw rounded to float): below 2K * 2.5e-7 + 4e-7; the margin is
-  // about four times that, and draws inside it read the exact entry.
+  // Error of the estimate below of u - t/2^32: 2^-23 for the draw cut to 23
+  // bits, 2^-22 for the hardware's 2^x, 2^-23 for the addition, and seven
+  // roundings of the exponent (2K, log2 e, two projections, three products),
+  // 2^-24 of a each, which e^-a turns into at most 2^-24 / e each: below
+  // 6.4e-7.  The margin is 24 times that and more, and draws inside it read
+  // the exact entry.
   const float margin = __fadd_rn(0x1p-16f, __fmul_rn(lat.twoK, 0x1p-20f));
   const float kexp = -__fmul_rn(lat.twoK, 0x1.715476p+0f);  // -2K log2 e
   const int mirror = (int)s_mirror;
