@@ -360,7 +360,7 @@ __device__ __forceinline__ void add_clock_sums(const Measure& mb, uint32_t slot_
 // Add a block's Potts histogram (shared bins) into its slot.
 __device__ __forceinline__ void add_histogram(const Lattice& lat, const Measure& mb, uint32_t slot_of,
                                               const unsigned int* s_hist) {
-  unsigned long long* slot = mb.hist + 256 * (slot_of % (uint32_t)hist_slots(lat.q));
+  unsigned long long* slot = mb.hist + 256 * (slot_of & (uint32_t)(hist_slots(lat.sbits) - 1));
   for (int k = threadIdx.x; k < lat.q; k += blockDim.x)
     if (s_hist[k]) atomicAdd(&slot[k], (unsigned long long)s_hist[k]);
 }
@@ -416,27 +416,33 @@ __device__ __forceinline__ void finalize_record(const Lattice& lat, const Measur
       mb.sums[2 * k + 1] = 0ull;
     }
     if (lat.model == kPotts) {
-      // n[k] = sum over slots, all (slot, k) pairs spread over the block, four
-      // loads in flight a thread
+      // n[k] = sum over slots, all (slot, k) pairs spread over the block: a
+      // load a thread, or four in flight
       __shared__ unsigned long long s_n[256];
       for (int k = threadIdx.x; k < 256; k += blockDim.x) s_n[k] = 0ull;
       __syncthreads();
-      const int cells = hist_slots(lat.q) * lat.q;
-      for (int t0 = threadIdx.x; t0 < cells; t0 += 4 * blockDim.x) {
-        int at[4];
-        unsigned long long v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int t = t0 + j * (int)blockDim.x;
-          at[j] = 256 * (t / lat.q) + t % lat.q;
-          v[j] = t < cells ? __ldcg(&mb.hist[at[j]]) : 0ull;
+      const int cells = hist_slots(lat.sbits) << lat.sbits, kmask = (1 << lat.sbits) - 1;
+      auto word = [&](int t) { return 256 * (t >> lat.sbits) + (t & kmask); };  // states past q hold 0
+      auto take = [&](int at, unsigned long long v) {
+        if (v) {
+          atomicAdd(&s_n[at & 255], v);
+          mb.hist[at] = 0ull;
         }
+      };
+      if (cells <= (int)blockDim.x) {
+        const int t = (int)threadIdx.x;
+        if (t < cells) take(word(t), __ldcg(&mb.hist[word(t)]));
+      } else {
+        for (int t0 = threadIdx.x; t0 < cells; t0 += 4 * blockDim.x) {
+          unsigned long long v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (v[j]) {
-            atomicAdd(&s_n[at[j] & 255], v[j]);
-            mb.hist[at[j]] = 0ull;
+          for (int j = 0; j < 4; ++j) {
+            const int t = t0 + j * (int)blockDim.x;
+            v[j] = t < cells ? __ldcg(&mb.hist[word(t)]) : 0ull;
           }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) take(word(t0 + j * (int)blockDim.x), v[j]);
+        }
       }
       __syncthreads();
       for (int k = threadIdx.x; k < lat.q; k += blockDim.x) g += (long long)(s_n[k] * s_n[k]);

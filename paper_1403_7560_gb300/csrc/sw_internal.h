@@ -62,24 +62,24 @@ inline void set_philox_key(Lattice& lat, uint64_t seed) {
 // single word takes an atomic from every block; the record is finalised by
 // one block of a later kernel in the same stream.
 constexpr int kSlots = 64;
-// Slots of the Potts histogram in use: fewer for many states, so that a
-// record's sum over slots and states is at most kHistCells words (each state
-// is a counter of its own, which spreads the blocks' additions as slots do).
+// Slots of the Potts histogram in use, by the bits of a state: fewer for many
+// states, so that a record's sum over slots and states is over at most
+// kHistCells words (each state is a counter of its own, which spreads the
+// blocks' additions as slots do).  A power of two, as the states are counted,
+// so that a word's slot and state are found without a division.
 // One CTA of 64 to 256 threads takes that sum, and the sweep waits for it: us
 // per sweep with 64 slots for any q / these, q = 256 (and q = 17, whose
 // lattice work is about the same): 2D L = 2048 95.9 / 35.9 (44.2 / 39.6),
 // a batch of one L = 1024 134.7 / 33.1 (43.1 / 35.3), of eight 3D L = 64
 // 144.6 / 37.8 (49.8 / 43.4).
 constexpr int kHistCells = 512;
-__host__ __device__ constexpr int hist_slots(int q) {
-  int s = kSlots;
-  while (s > 1 && s * q > kHistCells) s >>= 1;
-  return s;
+__host__ __device__ constexpr int hist_slots(int sbits) {
+  return (kHistCells >> sbits) < kSlots ? kHistCells >> sbits : kSlots;
 }
 struct Measure {
   unsigned long long* nclusters;  // roots counted by the flip kernel, [2][kSlots] by sweep parity
   unsigned long long* sums;       // [kSlots][2]: integer M, E (two's complement)
-  unsigned long long* hist;       // [kSlots][256]: Potts histogram (hist_slots(q) of the slots)
+  unsigned long long* hist;       // [kSlots][256]: Potts histogram (hist_slots of the slots)
   double* part_d;                 // XY per-block partials [3 * kMeasureBlocks]
   unsigned long long* csums;      // clock: [kSlots][3] integer sums of C[p_i], S[p_i], C[p_i - p_j]
   const long long* cfix;          // clock: C[p] = round(2^30 cos(2 pi p / q)) [q], then S [q]
