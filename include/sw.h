@@ -166,9 +166,9 @@ int sw_query(sw_handle* h);
 
 /* Failure-detection hook (no counterpart in the paper).  Every device loop
  * whose trip count depends on the data -- the union retries of the tile
- * labeling (shared memory) and of the global merge, the compression and
- * canonical-label walks, the label-equivalence walks and iterations of
- * sw_relabel -- is capped.  On valid input each ends far below the cap
+ * labeling (shared memory) and of the global merge, the walks of the
+ * compression, of the flip (up to 2^20 sites) and of the canonical labels,
+ * the label-equivalence walks and iterations of sw_relabel -- is capped.  On valid input each ends far below the cap
  * (parents only decrease), so the cap only turns a corrupted forest into an
  * error instead of a hang: a loop that reaches it writes SW_ERR_TIMEOUT to
  * the handle's device error flag and gives up, the kernel returns, and the
@@ -181,8 +181,7 @@ int sw_query(sw_handle* h);
  *              the error path without a fault)
  *   cap < 0    restores the production cap (2^22 steps)
  * Takes effect for launches enqueued after the call; a batch member runs
- * with the cap its handle had when the batch last captured its sweep (a
- * member joining or leaving, or a configuration change, recaptures it).
+ * with the cap its handle has at the sw_batch_sweep call.
  * Returns SW_ERR_BAD_ARG for a NULL handle or cap > 2^22. */
 int sw_set_loop_cap(sw_handle* h, long long cap);
 

@@ -69,9 +69,9 @@ constexpr int kSlots = 64;
 // so that a word's slot and state are found without a division.
 // One CTA of 64 to 256 threads takes that sum, and the sweep waits for it: us
 // per sweep with 64 slots for any q / these, q = 256 (and q = 17, whose
-// lattice work is about the same): 2D L = 2048 95.9 / 35.9 (44.2 / 39.6),
-// a batch of one L = 1024 134.7 / 33.1 (43.1 / 35.3), of eight 3D L = 64
-// 144.6 / 37.8 (49.8 / 43.4).
+// lattice work is about the same): 2D L = 2048 95.9 / 33.8 (44.2 / 39.3),
+// a batch of one L = 1024 134.7 / 31.4 (43.1 / 34.5), of eight 3D L = 64
+// 144.6 / 37.8 (49.8 / 42.0).
 constexpr int kHistCells = 512;
 __host__ __device__ constexpr int hist_slots(int sbits) {
   return (kHistCells >> sbits) < kSlots ? kHistCells >> sbits : kSlots;
@@ -271,11 +271,15 @@ size_t handle_block_bytes();
 // Small Ising/Potts lattices (sw_small.cu): whole sweeps by one CTA with
 // the lattice in shared memory, n sweeps per launch, records written as
 // the tiled path writes them.
-// the limits are where the one-CTA path stops beating the tiled one with its
-// split labeling (us per sweep at T_c, one CTA / tiled): 2D Ising L = 96 13.8 /
-// 18.8, 112 17.9 / 18.6, 128 19.5 / 20.4, 2D Potts q = 3 L = 128 23.4 / 22.7;
-// 3D Ising L = 18 14.4 / 23.8, 20 17.7 / 24.9 (beyond 22 the shared memory
-// does not hold it).
+// The limits are where the one-CTA path stops beating the tiled one with its
+// split labeling on a single lattice (us per sweep at T_c, one CTA / tiled):
+// 2D Ising L = 96 13.8 / 18.8, 112 17.9 / 18.6, 128 19.5 / 20.4, 2D Potts q =
+// 3 L = 128 23.4 / 22.7; 3D Ising L = 18 14.4 / 23.8, 20 17.7 / 24.9, 23 22.3 /
+// 21.1 (Potts of more than two states does not fit from 23 on).  In a batch
+// one CTA a member is the faster form up to them at every number of members
+// (us per batch sweep, one CTA / tiled): 64 of 2D L = 112 19.0 / 39.9, 600 99.0
+// / 110.7, 600 of L = 64 49.2 / 74.2, 64 of 3D L = 22 24.0 / 60.6, 600 109.2 /
+// 175.5, 600 of L = 16 66.5 / 78.4.
 constexpr uint32_t kSmallSites2D = 12544, kSmallSites3D = 10648;
 // Dynamic shared memory a small lattice may take (227 KB a CTA less the
 // static part).

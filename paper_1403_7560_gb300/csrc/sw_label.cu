@@ -25,9 +25,9 @@
 //   counts is instructions.  A union is two walks and an atomic in a loop the
 //   warp leaves with its slowest thread, so the hooks took the loop from 21 to
 //   8 trips a warp; four sites per thread share the row's loads, address
-//   arithmetic and one 16-byte store.  3D Ising L = 256 at T_c: 85.0 M -> 70.2
-//   M warp instructions, 108.9 -> 87.1 us; from bond planes (XY) 76.2 -> 59.3
-//   us; 2D L = 4096 94.8 -> 76.2 us; 3D L = 100 38.9 -> 29.1 us (ncu, cold L2).
+//   arithmetic and one 16-byte store.  3D Ising L = 256 at T_c: 85.0 M -> 67.4
+//   M warp instructions, 108.9 -> 85.4 us; from bond planes (XY) 76.2 -> 59.3
+//   us; 2D L = 4096 94.8 -> 76.2 us (ncu, cold L2).
 //   With MEASURE the row threads also measure the incoming spins (the state
 //   after the previous sweep) from the same bytes and equality masks.
 // k_bonds_xy: XY bonds: project on the sweep's mirror axis (once per site,
