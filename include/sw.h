@@ -306,7 +306,7 @@ size_t sw_series_capacity(void);
  * SW_BATCH_TILE_SHAPES shapes: 2D 32x256, 32x128, 32x64; 3D 32x16x16,
  * 32x16x8, 32x8x8 (single lattices use 32x128 in 2D, shape 1, and
  * 32x16x16 in 3D, shape 0, which a new batch starts with).  The schedule
- * (0 .. SW_BATCH_SCHEDULES - 1) has two bits.  Bit 0 is the label layout: 0
+ * (0 .. SW_BATCH_SCHEDULES - 1) has three bits.  Bit 0 is the label layout: 0
  * runs the Ising tiles in one launch with the two-state layout and the Potts
  * tiles in another, 1 runs all tiles in one launch with the Potts layout.
  * Bit 1 is the grid form of every phase (labels, merge, compression, apply):

@@ -220,7 +220,7 @@ cudaError_t launch_labels_out(const Lattice& lat, int32_t* out, cudaStream_t st)
 // Batched phases: one launch per phase over every tile of every member
 // (Ising/Potts, one dimension, tile shape `shape`), then the step counter
 // advances.  The tile map lists the Ising members' tiles first (ising_tiles
-// of them), then the Potts members' tiles.  A schedule has two bits:
+// of them), then the Potts members' tiles.  A schedule has three bits:
 //   bit 0 (label layout): 0 = the Ising tiles in one launch (two-state
 //     layout), the Potts tiles in another; 1 = every tile in one launch
 //     (Potts layout, the member's model picked per tile);

@@ -28,7 +28,7 @@
 // shared memory and written (with the FP64 accumulators, in sweep order)
 // every kRing sweeps by one warp.
 //   What bounds it is one warp's chain of instructions and the barriers (8
-// cycles from one instruction of a warp to its next, 47% of the SM's issue
+// cycles from one instruction of a warp to its next, 52% of the SM's issue
 // slots at L = 64), so work per phase was cut rather than spread.  us per
 // sweep, this kernel against a thread per site with byte states: 2D Ising L =
 // 64 13.3 -> 7.4, L = 90 21.5 -> 12.9, 3D L = 16 24.3 -> 11.4.  Listing the
